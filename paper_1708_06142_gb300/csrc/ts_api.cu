@@ -356,12 +356,14 @@ static ts_status ingest_mesh(ts_ctx* c, const ts_mesh* m) {
 
     std::vector<int> leaf_nid(nleaf);
     std::vector<double> leaf_lo(3 * (size_t)nleaf), leaf_size(3 * (size_t)nleaf);
+    c->min_edge = INFINITY;
     for (int n = 0; n < nleaf; ++n) {
         int b = c->leaf_blk[n];
         leaf_nid[n] = c->blk_nid[b];
         for (int a = 0; a < 3; ++a) {
             leaf_lo[3 * n + a] = m->lo[3 * b + a];
             leaf_size[3 * n + a] = m->size[3 * b + a];
+            c->min_edge = std::min(c->min_edge, leaf_size[3 * n + a] / TS_NB);
         }
     }
     cudaError_t e = cudaSuccess;

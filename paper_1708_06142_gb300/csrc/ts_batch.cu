@@ -55,7 +55,7 @@ __host__ __device__ inline size_t batch_warp_smem(int npix) {
 }
 
 // CLS: 0 gravity on isolated grids, 1 gravity on periodic/mixed grids, 2 columns
-template <int MAC, int CLS, int EWM = 2>
+template <int MAC, int CLS, int EWM = 2, bool SUB = false>
 __global__ void __launch_bounds__(32 * TS_WALK_WARPS) k_batch_walk(const __grid_constant__ BatchArgs A) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     __shared__ int64_t s_begin[TS_BATCH_MAX_SEG + 1];
@@ -105,8 +105,8 @@ __global__ void __launch_bounds__(32 * TS_WALK_WARPS) k_batch_walk(const __grid_
             if constexpr (CLS == 2)
                 col_walk_warp(W.cp, local, lane, map, W.com, W.cen, W.cstack, W.half, W.h2);
             else
-                walk_warp<float, CLS, MAC, false, 1, EWM>(W.wp, local, warp, lane, W.com, W.cen, W.cw, W.mask, W.half, W.h2,
-                                                     nullptr);
+                walk_warp<float, CLS, MAC, false, 1, EWM, false, SUB>(W.wp, local, warp, lane, W.com, W.cen, W.cw, W.mask,
+                                                                      W.half, W.h2, nullptr);
             __syncwarp();
         }
     }
@@ -257,18 +257,22 @@ static int periodic_kind(const int bc[3]) {
 }
 
 // One persistent launch of class CLS: as many CTAs as fit (or ctas_per_sm) on every SM.
-template <int MAC, int CLS, int EWM = 2>
+template <int MAC, int CLS, int EWM = 2, bool SUB = false>
 static cudaError_t launch_cls(ts_batch* b, const BatchArgs& A, cudaStream_t st) {
+    // a batch holding a mesh of extremely small cells keeps rsqrtf (see rsq)
+    if constexpr (CLS == 0 && !SUB)
+        for (size_t i = 0; i < b->ctx.size(); ++i)
+            if (b->h_wp[i].tiny) return launch_cls<MAC, CLS, EWM, true>(b, A, st);
     const size_t smem = TS_WALK_WARPS * batch_warp_smem(A.npix);
-    cudaError_t e = cudaFuncSetAttribute(k_batch_walk<MAC, CLS, EWM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_batch_walk<MAC, CLS, EWM, SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int nsm = 152, per = 1;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b->device);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch_walk<MAC, CLS, EWM>, 32 * TS_WALK_WARPS, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch_walk<MAC, CLS, EWM, SUB>, 32 * TS_WALK_WARPS, smem);
     if (b->ctas_per_sm > 0) per = std::min(per, b->ctas_per_sm);
     const int64_t need = (A.total + TS_WALK_WARPS - 1) / TS_WALK_WARPS;   // no idle CTAs for small classes
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)nsm * std::max(per, 1), need));
-    k_batch_walk<MAC, CLS, EWM><<<grid, 32 * TS_WALK_WARPS, smem, st>>>(A);
+    k_batch_walk<MAC, CLS, EWM, SUB><<<grid, 32 * TS_WALK_WARPS, smem, st>>>(A);
     return cudaGetLastError();
 }
 
@@ -493,6 +497,7 @@ extern "C" ts_status ts_batch_run(ts_batch* b, const ts_gravity_params* gp, void
                                  (uint64_t)(density != nullptr)};
     sig.push_back((uint64_t)b->mode);
     sig.push_back((uint64_t)b->nstreams);
+    for (int i = 0; i < n; ++i) sig.push_back((uint64_t)b->h_wp[i].tiny);   // chooses the kernel
     for (int i = 0; i < n; ++i) {
         sig.push_back(density ? (uint64_t)density[i] : 0);
         sig.push_back(gp ? (uint64_t)pot[i] : 0);

@@ -84,6 +84,7 @@ struct ts_ctx {
     int64_t ncell = 0;
     int bc[3] = {0, 0, 0};
     double L[3] = {1, 1, 1}, dlo[3] = {0, 0, 0};
+    double min_edge = 0;             // shortest cell edge of the mesh
     std::vector<int> blk_nid;        // node id of each block
     std::vector<int> leaf_blk;       // block of each leaf
     std::vector<int> amr_order;      // non-leaf node ids, deepest first

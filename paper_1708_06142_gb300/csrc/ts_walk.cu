@@ -69,6 +69,9 @@ cudaError_t make_walk_params(ts_ctx* c, const ts_gravity_params* p, void* pot, v
     P.leaf_begin = 0;
     P.leaf_end = c->nleaf;
     P.root_cw = c->root_cw;
+    // A nonzero separation is at least 2^-26 of the smallest cell edge (the FP32 spacing of cell
+    // centres), so from an edge of 1e-11 on no squared separation is below 2^-126.
+    P.tiny = c->min_edge < 1e-11 ? 1 : 0;
     P.theta2 = p->theta * p->theta;
     P.eta = p->safe_box;
     P.a_lim = p->a_lim;

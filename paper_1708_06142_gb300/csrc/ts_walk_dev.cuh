@@ -37,6 +37,7 @@ struct WalkParams {
     int64_t ncell;
     uint32_t root_cw;
     uint32_t sb_depths;   // bit d: the safe-box test can change a MAC decision for nodes at depth d
+    int tiny;             // 1: a squared separation of the mesh can be subnormal in FP32 (see rsq)
     double theta2, eta, a_lim, G, eps_rel;
     const float* a_old;
     const WalkGeom* geom;
@@ -69,6 +70,17 @@ __device__ __forceinline__ float rint_t(float x) { return rintf(x); }
 __device__ __forceinline__ double rint_t(double x) { return rint(x); }
 __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
+// 1/sqrt(x).  SUB = false: the hardware instruction alone, which flushes subnormal inputs.  rsqrtf
+// also rescales those, three more instructions on every call (24 of the ~200 of a popped group: the
+// 2M-cell Plummer BH walk ran 9 % longer with it); it is kept for meshes whose cells are so small
+// that a squared separation can be subnormal (WalkParams::tiny).  Normal inputs give the same bits.
+template <bool SUB>
+__device__ __forceinline__ float rsq(float x) {
+    if constexpr (SUB) return rsqrtf(x);
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 __device__ __forceinline__ float log_t(float x) { return logf(x); }
 __device__ __forceinline__ double log_t(double x) { return log(x); }
 
@@ -104,13 +116,14 @@ __device__ __forceinline__ void pk_sep(float2 cx, float2 cy, float2 cz, float2 n
 }
 
 // sums of m/|d| and m (c - r)/|d|^3 over the accepted children of the pair
+template <bool SUB>
 __device__ __forceinline__ void pk_interact(float2 dx, float2 dy, float2 dz, float2 d2, float2 m, bool a0, bool a1,
                                             float2& sp, float2& sx, float2& sy, float2& sz) {
     d2.x = a0 ? d2.x : 1.f;
     d2.y = a1 ? d2.y : 1.f;
     m.x = a0 ? m.x : 0.f;
     m.y = a1 ? m.y : 0.f;
-    const float2 inv = make_float2(rsqrtf(d2.x), rsqrtf(d2.y));
+    const float2 inv = make_float2(rsq<SUB>(d2.x), rsq<SUB>(d2.y));
     const float2 mi = __fmul2_rn(m, inv);
     sp = __fadd2_rn(sp, mi);
     const float2 g3 = __fmul2_rn(mi, __fmul2_rn(inv, inv));
@@ -121,11 +134,12 @@ __device__ __forceinline__ void pk_interact(float2 dx, float2 dy, float2 dz, flo
 
 // the same sums with a rejected child's d2 replaced by +inf: rsqrt(+inf) = 0, so it adds exactly 0
 // (its d2 may be 0: the target's own cell, or a node centred on the target)
+template <bool SUB>
 __device__ __forceinline__ void pk_interact_m(float2 dx, float2 dy, float2 dz, float2 d2, float2 m, bool a0, bool a1,
                                               float2& sp, float2& sx, float2& sy, float2& sz) {
     d2.x = a0 ? d2.x : __int_as_float(0x7f800000);   // +inf: rsqrt gives 0, the child adds nothing
     d2.y = a1 ? d2.y : __int_as_float(0x7f800000);
-    const float2 inv = make_float2(rsqrtf(d2.x), rsqrtf(d2.y));
+    const float2 inv = make_float2(rsq<SUB>(d2.x), rsq<SUB>(d2.y));
     const float2 mi = __fmul2_rn(m, inv);
     sp = __fadd2_rn(sp, mi);
     const float2 g3 = __fmul2_rn(mi, __fmul2_rn(inv, inv));
@@ -267,8 +281,9 @@ __device__ __forceinline__ R mimg(R d, int per, R L, R iL) {
 // stages only MPE moments), stack and masks, the depth geometry, and (learned-correction mode) the
 // network weights and this warp's row buffers.  POT: potential only (Sec. 2.2.2, eq. pot; the
 // acceleration is then obtained by numerical differentiation of the potential): the acceleration
-// sums are not formed and acc is not written.
-template <typename R, int BCK, int MAC, bool REL, int T, int EWM = 2, bool POT = false>
+// sums are not formed and acc is not written.  SUB (paired path): squared separations may be
+// subnormal (see rsq).
+template <typename R, int BCK, int MAC, bool REL, int T, int EWM = 2, bool POT = false, bool SUB = false>
 __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int warp, int lane,
                                           typename RT<R>::V4* s_com_w, typename RT<R>::V4* s_cen_w,
                                           uint32_t* s_cw_w, uint32_t (*s_mask_w)[T], const R (*s_half)[3],
@@ -426,7 +441,7 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
                             float2 cx, cy, cz, m, dx, dy, dz, d2;
                             pk_pair(X, Y, Z, M, h, cx, cy, cz, m);
                             pk_sep(cx, cy, cz, nrx, nry, nrz, dx, dy, dz, d2);
-                            pk_interact(dx, dy, dz, d2, m, true, true, sp, sax, say, saz);
+                            pk_interact<SUB>(dx, dy, dz, d2, m, true, true, sp, sax, say, saz);
                         }
                     }
                 } else {
@@ -440,7 +455,7 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
                             float2 cx, cy, cz, m, dx, dy, dz, d2;
                             pk_pair(X, Y, Z, M, h, cx, cy, cz, m);
                             pk_sep(cx, cy, cz, nrx, nry, nrz, dx, dy, dz, d2);
-                            pk_interact_m(dx, dy, dz, d2, m, j0 != self0, j0 + 1 != self0, sp, sax, say, saz);
+                            pk_interact_m<SUB>(dx, dy, dz, d2, m, j0 != self0, j0 + 1 != self0, sp, sax, say, saz);
                         }
                     }
                 }
@@ -544,17 +559,17 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
                 n_mac_w += 8u * lanes;
                 const float4* sx = P.ncom_soa + 8 * ((first - 1) >> 3);
                 float2 sp = make_float2(0.f, 0.f), sax = sp, say = sp, saz = sp;
+                const bool a_act = act[0];
                 // BH: accept iff d^2 > h^2 / theta^2, the threshold formed once per pop
-                const float hb = (float)h2 * ith2;
+                const float hb = a_act ? (float)h2 * ith2 : __int_as_float(0x7f800000);
                 const float2 hh = make_float2((float)h2, (float)h2);
                 const float2 gg = make_float2((float)G, (float)G), al = make_float2((float)alim[0], (float)alim[0]);
-                const bool a_act = act[0];
                 auto pairs = [&](unsigned ins) {
 #pragma unroll
                     for (int q = 0; q < 2; ++q) {
                         const float4 X = __ldg(sx + q), Y = __ldg(sx + 2 + q);
                         const float4 Z = __ldg(sx + 4 + q), M = __ldg(sx + 6 + q);
-                        uint32_t om[4];   // open masks of children 4 q .. 4 q + 3, parked by one store
+                        uint32_t om[4];   // accepting lanes of children 4 q .. 4 q + 3, parked by one store
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             const int j0 = 4 * q + 2 * h;
@@ -569,7 +584,7 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
                                 const float4* bq = (const float4*)s_bm_w;
                                 float2 b2, b3, bm, unused;
                                 pk_pair(bq[q], bq[2 + q], bq[4 + q], bq[4 + q], h, b2, b3, bm, unused);
-                                inv = make_float2(rsqrtf(d2.x), rsqrtf(d2.y));
+                                inv = make_float2(rsq<SUB>(d2.x), rsq<SUB>(d2.y));
                                 const float2 qq = __ffma2_rn(make_float2(-bm.x, -bm.y), inv, make_float2(1.f, 1.f));
                                 const float2 i2 = __fmul2_rn(inv, inv);
                                 const float2 br = __ffma2_rn(__fmul2_rn(make_float2(3.f, 3.f), b2), i2,
@@ -579,22 +594,22 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
                                 const float2 rhs = __fmul2_rn(__fmul2_rn(al, qq), qq);
                                 mac0 = qq.x > 0.f && lhs.x < rhs.x; mac1 = qq.y > 0.f && lhs.y < rhs.y;
                             } else if constexpr (MAC == TS_MAC_BH) {
-                                mac0 = d2.x > hb; mac1 = d2.y > hb;
+                                mac0 = d2.x > hb; mac1 = d2.y > hb;   // (hb infinite in lanes outside the mask)
                             } else {
                                 const float2 lhs = __fmul2_rn(__fmul2_rn(gg, m), hh);
                                 const float2 rhs = __fmul2_rn(__fmul2_rn(al, d2), d2);
                                 mac0 = lhs.x < rhs.x; mac1 = lhs.y < rhs.y;
                             }
-                            const bool a0 = a_act && mac0 && !((ins >> j0) & 1u);
-                            const bool a1 = a_act && mac1 && !((ins >> (j0 + 1)) & 1u);
-                            om[2 * h] = __ballot_sync(0xffffffffu, a_act && !a0);
-                            om[2 * h + 1] = __ballot_sync(0xffffffffu, a_act && !a1);
+                            const bool a0 = (MAC == TS_MAC_BH || a_act) && mac0 && !((ins >> j0) & 1u);
+                            const bool a1 = (MAC == TS_MAC_BH || a_act) && mac1 && !((ins >> (j0 + 1)) & 1u);
+                            om[2 * h] = __ballot_sync(0xffffffffu, a0);
+                            om[2 * h + 1] = __ballot_sync(0xffffffffu, a1);
                             // (no warp vote to skip pairs nobody accepts: most children are
                             // accepted, and the vote costs more than it saves)
                             if constexpr (MAC == TS_MAC_MPE)
                                 pk_interact_inv(dx, dy, dz, inv, m, a0, a1, sp, sax, say, saz);
                             else
-                                pk_interact_m(dx, dy, dz, d2, m, a0, a1, sp, sax, say, saz);
+                                pk_interact_m<SUB>(dx, dy, dz, d2, m, a0, a1, sp, sax, say, saz);
                         }
                         if (lane == 0)
                             *(uint4*)&s_mask_w[TS_WALK_STACK - 8 + 4 * q][0] = make_uint4(om[0], om[1], om[2], om[3]);
@@ -667,6 +682,7 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
             __syncwarp();
 #pragma unroll
             for (int t = 0; t < T; ++t) my_om[t] = lane < 8 ? s_mask_w[TS_WALK_STACK - 8 + lane][t] : 0u;
+            if constexpr (PK) my_om[0] = lane < 8 ? m0 & ~my_om[0] : 0u;   // (the paired path parks who accepts)
             // (the paired path counts its accepted pairs at the end, from the pops' lane counts)
             // push the opened children in one compacted write: lane j < 8 owns child j
             bool mine = false;

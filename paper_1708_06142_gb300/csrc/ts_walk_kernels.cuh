@@ -13,7 +13,7 @@ struct WalkMinBlocks {
     static constexpr int value = (sizeof(R) == 4 && BCK == 0 && MAC == TS_MAC_BH && T == 1) ? 7 : 1;
 };
 
-template <typename R, int BCK, int MAC, bool REL, int T, int EWM, bool POT = false>
+template <typename R, int BCK, int MAC, bool REL, int T, int EWM, bool POT = false, bool SUB = false>
 __global__ void __launch_bounds__(32 * TS_WALK_WARPS, (WalkMinBlocks<R, BCK, MAC, T>::value))
     k_gravity_walk(const __grid_constant__ WalkParams P) {
     typedef typename RT<R>::V4 V4;
@@ -56,12 +56,15 @@ __global__ void __launch_bounds__(32 * TS_WALK_WARPS, (WalkMinBlocks<R, BCK, MAC
         gw += P.leaf_begin * (16 / T);           // 16 / T warps per leaf-block of 512 cells
         if (gw * 32 * T >= P.leaf_end * 512) return;
     }
-    walk_warp<R, BCK, MAC, REL, T, EWM, POT>(P, gw, warp, lane, s_com[warp], s_cen[warp], s_cw[warp], s_mask[warp], s_half,
-                                        s_h2, s_dyn, s_bm[MAC == TS_MAC_MPE ? warp : 0]);
+    walk_warp<R, BCK, MAC, REL, T, EWM, POT, SUB>(P, gw, warp, lane, s_com[warp], s_cen[warp], s_cw[warp], s_mask[warp],
+                                                  s_half, s_h2, s_dyn, s_bm[MAC == TS_MAC_MPE ? warp : 0]);
 }
 
-template <typename R, int BCK, int MAC, bool REL, int T, int EWM = 2, bool POT = false>
+template <typename R, int BCK, int MAC, bool REL, int T, int EWM = 2, bool POT = false, bool SUB = false>
 static cudaError_t launch_t(ts_ctx* c, const WalkParams& P) {
+    // the paired walk of a mesh of extremely small cells keeps rsqrtf (see rsq)
+    if constexpr (sizeof(R) == 4 && BCK == 0 && T == 1 && !SUB)
+        if (P.tiny) return launch_t<R, BCK, MAC, REL, T, EWM, POT, true>(c, P);
     // warp lists: an upper bound
     const int64_t nwarps = P.targets ? P.ntargets / 32 : (P.leaf_end - P.leaf_begin) * (16 / T);
     if (nwarps <= 0) return cudaSuccess;
@@ -69,11 +72,11 @@ static cudaError_t launch_t(ts_ctx* c, const WalkParams& P) {
     size_t smem = 0;
     if constexpr (BCK == 2) {
         smem = MLP_SMEM_WEIGHTS + TS_WALK_WARPS * MLP_SMEM_WARP;
-        cudaError_t e = cudaFuncSetAttribute(k_gravity_walk<R, BCK, MAC, REL, T, EWM, POT>,
+        cudaError_t e = cudaFuncSetAttribute(k_gravity_walk<R, BCK, MAC, REL, T, EWM, POT, SUB>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k_gravity_walk<R, BCK, MAC, REL, T, EWM, POT><<<grid, 32 * TS_WALK_WARPS, smem, c->stream>>>(P);
+    k_gravity_walk<R, BCK, MAC, REL, T, EWM, POT, SUB><<<grid, 32 * TS_WALK_WARPS, smem, c->stream>>>(P);
     return cudaGetLastError();
 }
 
