@@ -541,7 +541,7 @@ extern "C" ts_status ts_ewald_field(ts_ctx* c, int32_t n, const char* cache_path
     cudaError_t e = cudaSuccess;
     auto chk = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
     chk(dalloc(c->d_ew64, npts));
-    chk(dalloc(c->d_ew32, npts));
+    chk(dalloc(c->d_ew32, 2 * npts));
     if (e != cudaSuccess) { free_ewald(c); return ts_cuda_fail(e, "ts_ewald_field: allocation"); }
     if (loaded) {
         chk(cudaMemcpyAsync(c->d_ew64, c->ew_host.data(), sizeof(dbl4) * npts, cudaMemcpyHostToDevice, c->stream));
@@ -553,11 +553,7 @@ extern "C" ts_status ts_ewald_field(ts_ctx* c, int32_t n, const char* cache_path
     if (e != cudaSuccess) { free_ewald(c); return ts_cuda_fail(e, "ts_ewald_field: table generation"); }
     for (size_t i = 0; i < npts * 4; ++i)
         if (!isfinite(c->ew_host[i])) { free_ewald(c); return ts_fail(TS_ERR_NUMERIC, "ts_ewald_field: non-finite table value"); }
-    std::vector<float4> t32(npts);
-    for (size_t i = 0; i < npts; ++i)
-        t32[i] = make_float4((float)c->ew_host[4 * i], (float)c->ew_host[4 * i + 1], (float)c->ew_host[4 * i + 2],
-                             (float)c->ew_host[4 * i + 3]);
-    chk(cudaMemcpyAsync(c->d_ew32, t32.data(), sizeof(float4) * npts, cudaMemcpyHostToDevice, c->stream));
+    chk(launch_ewald_pairs(c, n, c->d_ew64, c->d_ew32));
     chk(cudaStreamSynchronize(c->stream));
     if (e != cudaSuccess) { free_ewald(c); return ts_cuda_fail(e, "ts_ewald_field: upload"); }
     if (cache_path && !loaded) {
@@ -631,7 +627,8 @@ ts_status ensure_taylor(ts_ctx* c) {
         o[4] = r[4]; o[5] = r[7]; o[6] = r[8]; o[7] = r[5]; o[8] = r[9]; o[9] = r[6];
         // 32-byte record: (C, A_c) in FP32, then (Jxx, Jyy), (Jzz, Jxy), (Jxz, Jyz) as FP16 pairs of
         // J / s and s = max |J| in the last word
-        t32[2 * i] = make_float4((float)r[0], (float)r[1], (float)r[2], (float)r[3]);
+        const size_t o32 = 2 * ((i % n * n + i / n % n) * n + i / n / n);   // x fastest
+        t32[o32] = make_float4((float)r[0], (float)r[1], (float)r[2], (float)r[3]);
         double s = 0;
         for (int k = 4; k < 10; ++k) s = std::max(s, fabs(r[k]));
         if (!(s > 0)) s = 1;
@@ -647,7 +644,7 @@ ts_status ensure_taylor(ts_ctx* c) {
         pk.y = h16(r[6]) | (h16(r[7]) << 16);
         pk.z = h16(r[8]) | (h16(r[9]) << 16);
         memcpy(&pk.w, &sf, 4);
-        memcpy(&t32[2 * i + 1], &pk, 16);
+        memcpy(&t32[o32 + 1], &pk, 16);
     }
     chk(cudaMemcpyAsync(c->d_tay32, t32.data(), sizeof(float4) * t32.size(), cudaMemcpyHostToDevice, c->stream));
     chk(cudaStreamSynchronize(c->stream));

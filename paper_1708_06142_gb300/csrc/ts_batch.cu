@@ -260,7 +260,7 @@ static int periodic_kind(const int bc[3]) {
 template <int MAC, int CLS, int EWM = 2, bool SUB = false>
 static cudaError_t launch_cls(ts_batch* b, const BatchArgs& A, cudaStream_t st) {
     // a batch holding a mesh of extremely small cells keeps rsqrtf (see rsq)
-    if constexpr (CLS == 0 && !SUB)
+    if constexpr (CLS <= 1 && !SUB)
         for (size_t i = 0; i < b->ctx.size(); ++i)
             if (b->h_wp[i].tiny) return launch_cls<MAC, CLS, EWM, true>(b, A, st);
     const size_t smem = TS_WALK_WARPS * batch_warp_smem(A.npix);

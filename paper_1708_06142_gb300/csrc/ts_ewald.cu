@@ -205,6 +205,24 @@ __global__ void k_ewald_table(EwGen g, double* __restrict__ out) {
     }
 }
 
+// FP32 trilinear records of the table (EwaldDev::tab32): (C, A_c) of point (i, j, k) and of (i + 1, j, k),
+// x fastest; the last point of a row repeats itself (its record is never read).
+__global__ void k_ewald_pairs(int n, const dbl4* __restrict__ tab, float4* __restrict__ out) {
+    const int64_t npts = (int64_t)n * n * n;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < npts; t += (int64_t)gridDim.x * blockDim.x) {
+        const int i = (int)(t % n), j = (int)((t / n) % n), k = (int)(t / ((int64_t)n * n));
+        const dbl4 a = tab[((int64_t)i * n + j) * n + k], b = tab[((int64_t)min(i + 1, n - 1) * n + j) * n + k];
+        out[2 * t] = make_float4((float)a.x, (float)a.y, (float)a.z, (float)a.w);
+        out[2 * t + 1] = make_float4((float)b.x, (float)b.y, (float)b.z, (float)b.w);
+    }
+}
+
+cudaError_t launch_ewald_pairs(ts_ctx* c, int n, const dbl4* tab64, float4* out) {
+    const int64_t npts = (int64_t)n * n * n;
+    k_ewald_pairs<<<(int)((npts + 255) / 256), 256, 0, c->stream>>>(n, tab64, out);
+    return cudaGetLastError();
+}
+
 // First-order Taylor table (Sec. 2.2.5, approach 2): at every grid point the correction and the
 // Jacobian J_ij = dA_c,i/dd_j of its acceleration part by central differences of the series with
 // step eps (A_c is a gradient field, so J is symmetrised).  Records of 4 dbl4 per point:

@@ -59,11 +59,13 @@ struct EwaldDev {
     double far_slope;          // 2P1I: 2 pi / (b Lx^2)
     double far_const;          // 2P1I: 2 sqrt(pi zeta)/(pi b Lx);  1P2I: -(gamma_E - ln 4 zeta)/Lx
     double far_lx;             // Lx
+    // trilinear table.  FP64: (C, A_c) per point, z fastest.  FP32: 32-byte records, x fastest, holding
+    // (C, A_c) of the point and of its neighbour at x + 1 (one 256-bit load per row of a table cell)
     const float4* tab32;
     const dbl4* tab64;
     // first-order Taylor table (Sec. 2.2.5, approach 2), J = dA_c/dd.  FP64: per grid point 4
     // records of 4 values, (C, A_cx, A_cy, A_cz), (Jxx, Jyy, Jzz, Jxy), (Jxz, Jyz, 0, 0), (0, 0, 0, 0).
-    // FP32: per grid point 2 records, (C, A_c) and the FP16 pairs (Jxx, Jyy), (Jzz, Jxy), (Jxz, Jyz)
+    // FP32: per grid point (x fastest) one 32-byte record, (C, A_c) and the FP16 pairs (Jxx, Jyy), (Jzz, Jxy), (Jxz, Jyz)
     // of J / s with s = max |J| as the fourth word
     int taylor;                // 1: the walk expands about the nearest grid point instead of trilinear
     double h[3];               // grid spacing ext / (n - 1)
@@ -239,6 +241,7 @@ cudaError_t launch_zero_mean(ts_ctx* c, int precision, void* pot);
 cudaError_t launch_num_diff(ts_ctx* c, int precision, const void* pot, void* acc);
 ts_status ensure_numdiff(ts_ctx* c);
 cudaError_t launch_ewald_table(ts_ctx* c, int n, double* d_out64);
+cudaError_t launch_ewald_pairs(ts_ctx* c, int n, const dbl4* tab64, float4* out);
 cudaError_t launch_ewald_taylor(ts_ctx* c, int n, double eps, dbl4* d_out);
 ts_status ensure_taylor(ts_ctx* c);
 cudaError_t launch_noderay_dense(ts_ctx* c, int nside, const int dims[3], double psi_min,

@@ -51,6 +51,22 @@ static cudaError_t upload_geom(ts_ctx* c, WalkGeom** out) {
     return cudaMemcpyAsync(c->d_geom, &c->geom, sizeof(WalkGeom), cudaMemcpyHostToDevice, c->stream);
 }
 
+// The largest x with !(h2 < theta2 x) in FP32: the scalar form of the BH test, h2 < theta2 d^2, as one
+// comparison d^2 > x with the same decision for every d^2 (the product is monotonic in x).
+static float bh_threshold(float theta2, float h2) {
+    uint32_t lo = 0, hi = 0x7f800000u;   // +0 .. +inf: the bits order like the values
+    while (lo < hi) {
+        const uint32_t mid = lo + (hi - lo + 1) / 2;
+        float x;
+        memcpy(&x, &mid, 4);
+        volatile float q = theta2 * x;
+        if (!(h2 < q)) lo = mid; else hi = mid - 1;
+    }
+    float x;
+    memcpy(&x, &lo, 4);
+    return x;
+}
+
 // Kernel parameters of one context's walk (also used for the batched persistent kernel).
 // bck: 0 isolated, 1 correction table, 2 learned correction.
 cudaError_t make_walk_params(ts_ctx* c, const ts_gravity_params* p, void* pot, void* acc, WalkParams* out, int* bck_out) {
@@ -118,6 +134,21 @@ cudaError_t make_walk_params(ts_ctx* c, const ts_gravity_params* p, void* pot, v
     } else if (bck) {
         P.ew = c->ew;
         P.ew.taylor = p->ewald == TS_EWALD_TAYLOR ? 1 : 0;
+        EwF32& F = P.ef;
+        F.kind = P.ew.kind;
+        F.n = P.ew.n;
+        for (int a = 0; a < 3; ++a) { F.inv_dx[a] = (float)P.ew.inv_dx[a]; F.h[a] = (float)P.ew.h[a]; }
+        F.cap = P.ew.taylor ? F.n - 0.5f : F.n - 1.f;
+        F.far = (float)P.ew.far;
+        F.far_slope = (float)P.ew.far_slope;
+        F.far_const = (float)P.ew.far_const;
+        F.lx = (float)P.ew.far_lx;
+        F.two_over_lx = (float)(2.0 / P.ew.far_lx);
+        F.twopi_over_lx = (float)(2.0 * M_PI / P.ew.far_lx);
+        F.bias = 0x4b000000u * (uint32_t)(F.n * F.n + F.n + 1);
+        F.rec = (const float4*)((uintptr_t)(P.ew.taylor ? P.ew.tay32 : P.ew.tab32) - (uintptr_t)F.bias * 32u);
+        if (p->mac == TS_MAC_BH)
+            for (int d = 0; d <= TS_MAX_DEPTH; ++d) P.thr[d] = bh_threshold((float)P.theta2, c->geom.hmax2_32[d]);
     }
     P.pot = pot;
     P.acc = acc;

@@ -28,6 +28,21 @@ struct RT<double> {
     typedef dbl4 V4;
 };
 
+// Correction lookup of the paired FP32 walk (periodic and mixed BCs): the FP32 values of EwaldDev.
+struct EwF32 {
+    int kind, n;
+    float inv_dx[3], h[3];
+    float cap;                        // largest scaled coordinate: n - 1/2 (Taylor), n - 1 (trilinear)
+    float far, far_slope, far_const;
+    float lx, two_over_lx, twopi_over_lx;
+    // 32-byte records, x fastest (EwaldDev::tay32 or tab32).  The index is formed from the bits of
+    // 2^23 + coordinate, 0x4b000000 + i: its constant part, bias = 0x4b000000 (n^2 + n + 1) mod 2^32,
+    // has its low 24 bits zero and the index is below 2^24, so the sum never wraps and rec points
+    // bias records before the table.
+    const float4* rec;
+    uint32_t bias;
+};
+
 struct WalkParams {
     const void* ncom;
     const void* ncen;
@@ -56,6 +71,8 @@ struct WalkParams {
     int64_t leaf_begin, leaf_end;
     unsigned long long* blk_counts;   // nullable: interactions per leaf-block (warp-list and full walks)
     EwaldDev ew;
+    EwF32 ef;
+    float thr[TS_MAX_DEPTH + 1];      // paired periodic BH walk: accept iff d^2 > thr[depth]
     void* pot;
     void* acc;
     int* status;
@@ -213,7 +230,7 @@ __device__ __forceinline__ void ewald_pair(const EwaldDev& E, R dx, R dy, R dz, 
         if constexpr (sizeof(R) == 4) {
             // one 32-byte record (one L1 sector): (C, A_c), then the Jacobian as FP16 pairs of J / s
             // (Jxx, Jyy), (Jzz, Jxy), (Jxz, Jyz) and s; the displacement is scaled by s instead
-            const float4* rec = (const float4*)E.tay32 + 2 * (((size_t)g0 * n + g1) * n + g2);
+            const float4* rec = (const float4*)E.tay32 + 2 * (((size_t)g2 * n + g1) * n + g0);
             const float4 v = __ldg(rec);
             const uint4 q = __ldg((const uint4*)rec + 1);
             const float s = __uint_as_float(q.w);
@@ -249,14 +266,14 @@ __device__ __forceinline__ void ewald_pair(const EwaldDev& E, R dx, R dy, R dz, 
         i0[a] = i;
         f[a] = v - (R)i;
     }
-    const V4* tab;
-    if constexpr (sizeof(R) == 4) tab = (const V4*)E.tab32; else tab = (const V4*)E.tab64;
     R c = 0, cx = 0, cy = 0, cz = 0;
 #pragma unroll
     for (int o = 0; o < 8; ++o) {
         const int ox = o & 1, oy = (o >> 1) & 1, oz = o >> 2;
         const R w = (ox ? f[0] : (R)1 - f[0]) * (oy ? f[1] : (R)1 - f[1]) * (oz ? f[2] : (R)1 - f[2]);
-        const V4 v = tab[((size_t)(i0[0] + ox) * n + (i0[1] + oy)) * n + (i0[2] + oz)];
+        V4 v;
+        if constexpr (sizeof(R) == 4) v = E.tab32[2 * (((size_t)(i0[2] + oz) * n + (i0[1] + oy)) * n + i0[0]) + ox];
+        else v = E.tab64[((size_t)(i0[0] + ox) * n + (i0[1] + oy)) * n + (i0[2] + oz)];
         c += w * v.x; cx += w * v.y; cy += w * v.z; cz += w * v.w;
     }
     const R inv3 = inv * inv * inv;
@@ -265,6 +282,154 @@ __device__ __forceinline__ void ewald_pair(const EwaldDev& E, R dx, R dy, R dz, 
     Ax = dx * inv3 + (dx < (R)0 ? -cx : cx);
     Ay = dy * inv3 + (dy < (R)0 ? -cy : cy);
     Az = dz * inv3 + (dz < (R)0 ? -cz : cz);
+}
+
+// 32-byte record by one 256-bit load.  Measured on GB300 with scattered addresses: a 128-bit load
+// costs the L1 one cycle per distinct 128-byte line of the warp, a 256-bit load half a cycle per
+// distinct line of each group of 4 lanes, so a record costs half or less of two 128-bit loads.
+__device__ __forceinline__ void ld_rec(const float4* p, float4& a, float4& b) {
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+        : "l"(p));
+}
+
+// t with its sign flipped where d is negative (A_c is odd in its own axis)
+__device__ __forceinline__ float flip(float t, float d) {
+    return __uint_as_float(__float_as_uint(t) ^ (__float_as_uint(d) & 0x80000000u));
+}
+
+__device__ __forceinline__ float2 lerp2(float2 a, float2 b, float2 f) {
+    return __ffma2_rn(f, __ffma2_rn(a, make_float2(-1.f, -1.f), b), a);
+}
+
+// Minimum image of two separations at once: d - L rint(d / L), the rounding to the nearest integer by
+// adding and subtracting 1.5 * 2^23 (exact below 2^22; two packed additions where rintf needs the
+// conversion unit for each value).  An isolated axis has 1 / L = L = 0.
+__device__ __forceinline__ float2 pk_image(float2 d, float2 iL, float2 nL) {
+    const float2 M = make_float2(12582912.f, 12582912.f), N = make_float2(-12582912.f, -12582912.f);
+    return __ffma2_rn(__fadd2_rn(__fadd2_rn(__fmul2_rn(d, iL), M), N), nL, d);
+}
+
+// d^2 as the scalar kernels form it, fma(dx, dx, dy dy) + dz dz with the last product rounded by
+// itself, so that every MAC decision is theirs bit for bit.  (The last addition is scalar: a packed
+// one is fused with the packed product.)
+__device__ __forceinline__ float2 pk_norm2(float2 dx, float2 dy, float2 dz) {
+    const float2 a = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)), b = __fmul2_rn(dz, dz);
+    return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
+}
+
+// The paired periodic walk's lookup of a pair of children of which this lane accepts acc[0] and/or
+// acc[1]: adds m phi(d) and m A(d) of the separations d (their minimum images, child minus target) to
+// s01 = (phi, A_x) and s23 = (A_y, A_z); a child it does not accept adds nothing and reads record 0.
+// Both children's records are loaded before the first is used: the walk waits for these loads more
+// than for anything else (one child at a time: 16.6 ms on the 64^3 Taylor disk, both 14.7 ms).  The
+// grid point or cell index comes from adding 2^23 rounded down, whose bits hold the floor: two
+// integer multiply-adds on the bits make the record index, and no value passes through the
+// conversion unit.  The coordinates are clamped to the table before that, so any separation (also a
+// NaN) stays inside it.
+template <int EWM, bool POT, bool SUB>
+__device__ __forceinline__ void ew_pair(const EwF32& E, float2 px, float2 py, float2 pz, float2 pd2, float2 pm, bool a0,
+                                        bool a1, float2& s01, float2& s23) {
+    constexpr int N = 2;
+    const float dx[N] = {px.x, px.y}, dy[N] = {py.x, py.y}, dz[N] = {pz.x, pz.y};
+    const float d2[N] = {pd2.x, pd2.y}, m[N] = {pm.x, pm.y};
+    bool acc[N] = {a0, a1};
+    if (E.kind != TS_EW_3P) {
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            if (E.kind == TS_EW_2P1I) {
+                if (acc[u] && fabsf(dz[u]) > E.far) {
+                    s01.x = fmaf(m[u], E.far_const - E.far_slope * fabsf(dz[u]), s01.x);
+                    if constexpr (!POT) s23.y = fmaf(m[u], flip(E.far_slope, dz[u]), s23.y);
+                    acc[u] = false;
+                }
+            } else {
+                const float r2 = dy[u] * dy[u] + dz[u] * dz[u];
+                if (acc[u] && r2 > E.far * E.far) {
+                    s01.x = fmaf(m[u], E.far_const - E.two_over_lx * logf(E.twopi_over_lx * sqrtf(r2)), s01.x);
+                    if constexpr (!POT) {
+                        const float k = m[u] * 2.f / (E.lx * r2);
+                        s23.x = fmaf(k, dy[u], s23.x);
+                        s23.y = fmaf(k, dz[u], s23.y);
+                    }
+                    acc[u] = false;
+                }
+            }
+        }
+    }
+    constexpr float M23 = 8388608.f;
+    constexpr int NR = EWM == 1 ? 1 : 4;    // records of a child
+    const uint32_t n = (uint32_t)E.n;
+    float X[N], Y[N], Z[N], vx[N], vy[N], vz[N];
+    float4 ra[N][NR], rb[N][NR];
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        const float ax = fabsf(dx[u]), ay = fabsf(dy[u]), az = fabsf(dz[u]);
+        if constexpr (EWM == 1) {   // nearest grid point
+            X[u] = __fadd_rd(fminf(fmaf(ax, E.inv_dx[0], 0.5f), E.cap), M23);
+            Y[u] = __fadd_rd(fminf(fmaf(ay, E.inv_dx[1], 0.5f), E.cap), M23);
+            Z[u] = __fadd_rd(fminf(fmaf(az, E.inv_dx[2], 0.5f), E.cap), M23);
+        } else {   // lower corner of the cell; a coordinate on the upper edge takes the last cell
+            const float last = E.cap - 1.f;
+            vx[u] = fminf(ax * E.inv_dx[0], E.cap);
+            vy[u] = fminf(ay * E.inv_dx[1], E.cap);
+            vz[u] = fminf(az * E.inv_dx[2], E.cap);
+            X[u] = __fadd_rd(fminf(vx[u], last), M23);
+            Y[u] = __fadd_rd(fminf(vy[u], last), M23);
+            Z[u] = __fadd_rd(fminf(vz[u], last), M23);
+        }
+        uint32_t i = (__float_as_uint(Z[u]) * n + __float_as_uint(Y[u])) * n + __float_as_uint(X[u]);
+        i = acc[u] ? i : E.bias;
+        const float4* r = E.rec + 2 * (size_t)i;
+        ld_rec(r, ra[u][0], rb[u][0]);
+        if constexpr (EWM == 0) {   // (x, x + 1) at (y + 1, z), (y, z + 1), (y + 1, z + 1)
+            ld_rec(r + 2 * n, ra[u][1], rb[u][1]);
+            ld_rec(r + 2 * n * n, ra[u][2], rb[u][2]);
+            ld_rec(r + 2 * n * n + 2 * n, ra[u][3], rb[u][3]);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        const float inv = rsq<SUB>(acc[u] ? d2[u] : __int_as_float(0x7f800000));
+        const float mu = acc[u] ? m[u] : 0.f;
+        float c, tx = 0.f, ty = 0.f, tz = 0.f;
+        if constexpr (EWM == 1) {
+            const float4 v = ra[u][0], q = rb[u][0];
+            const float ux = fmaf(M23 - X[u], E.h[0], fabsf(dx[u])), uy = fmaf(M23 - Y[u], E.h[1], fabsf(dy[u])),
+                        uz = fmaf(M23 - Z[u], E.h[2], fabsf(dz[u]));
+            c = v.x - fmaf(v.w, uz, fmaf(v.z, uy, v.y * ux));
+            if constexpr (!POT) {
+                const uint32_t qx = __float_as_uint(q.x), qy = __float_as_uint(q.y), qz = __float_as_uint(q.z);
+                const float2 a = __half22float2(*(const __half2*)&qx), b = __half22float2(*(const __half2*)&qy),
+                             d = __half22float2(*(const __half2*)&qz);
+                const float sx = q.w * ux, sy = q.w * uy, sz = q.w * uz;
+                tx = fmaf(d.x, sz, fmaf(b.y, sy, fmaf(a.x, sx, v.y)));
+                ty = fmaf(d.y, sz, fmaf(a.y, sy, fmaf(b.y, sx, v.z)));
+                tz = fmaf(b.x, sz, fmaf(d.y, sy, fmaf(d.x, sx, v.w)));
+            }
+        } else {
+            const float fx = vx[u] - (X[u] - M23), fy = vy[u] - (Y[u] - M23), fz = vz[u] - (Z[u] - M23);
+            const float2 f2 = make_float2(fx, fx), g2 = make_float2(fy, fy), h2 = make_float2(fz, fz);
+            auto lo = [](const float4& w) { return make_float2(w.x, w.y); };
+            auto hi = [](const float4& w) { return make_float2(w.z, w.w); };
+            const float2 l = lerp2(lerp2(lerp2(lo(ra[u][0]), lo(rb[u][0]), f2), lerp2(lo(ra[u][1]), lo(rb[u][1]), f2), g2),
+                                   lerp2(lerp2(lo(ra[u][2]), lo(rb[u][2]), f2), lerp2(lo(ra[u][3]), lo(rb[u][3]), f2), g2), h2);
+            c = l.x;
+            if constexpr (!POT) {
+                const float2 w = lerp2(lerp2(lerp2(hi(ra[u][0]), hi(rb[u][0]), f2), lerp2(hi(ra[u][1]), hi(rb[u][1]), f2), g2),
+                                       lerp2(lerp2(hi(ra[u][2]), hi(rb[u][2]), f2), lerp2(hi(ra[u][3]), hi(rb[u][3]), f2), g2), h2);
+                tx = l.y; ty = w.x; tz = w.y;
+            }
+        }
+        if constexpr (POT) {
+            s01.x = fmaf(mu, inv + c, s01.x);
+        } else {
+            const float inv3 = inv * (inv * inv);
+            const float2 m2 = make_float2(mu, mu);
+            s01 = __ffma2_rn(m2, make_float2(inv + c, fmaf(dx[u], inv3, flip(tx, dx[u]))), s01);
+            s23 = __ffma2_rn(m2, make_float2(fmaf(dy[u], inv3, flip(ty, dy[u])), fmaf(dz[u], inv3, flip(tz, dz[u]))), s23);
+        }
+    }
 }
 
 // Minimum image along one axis (periodic axes only).
@@ -295,11 +460,15 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
     const V4* ncen = (const V4*)P.ncen;
     const V4* cell = (const V4*)P.cell;
     const int64_t base = gw * 32 * T;             // first Morton cell id of this warp
-    // the paired FP32 path: isolated FP32 walk with one target per lane (see below)
-    constexpr bool PK = sizeof(R) == 4 && BCK == 0 && T == 1;
+    // the paired FP32 path: FP32 walk with one target per lane and no learned correction (see below)
+    constexpr bool PK = sizeof(R) == 4 && BCK <= 1 && T == 1;
+    constexpr bool PKE = PK && BCK == 1;   // with the minimum image and the correction lookup
     // unrolling of the per-child loops of the scalar path: with the correction-table lookup inlined
     // into both, a 4-way unroll keeps the kernel body small enough for the instruction cache
     // (measured on the 3P 128^3 box: Taylor 28.6 -> 24.6 ms, trilinear 67.0 -> 58.4 ms)
+    // (the paired periodic walk: its quads of children are not unrolled at all; unrolled, 18.3 ms on the
+    // 64^3 Taylor disk against 16.2 ms)
+    constexpr int QUAD_UNROLL = PKE ? 1 : 2;
     constexpr int CHILD_UNROLL = BCK == 1 ? 4 : 8;
 
     R rx[T], ry[T], rz[T], alim[T];
@@ -311,7 +480,11 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
     const R iLx = (R)P.geom->invL[0], iLy = (R)P.geom->invL[1], iLz = (R)P.geom->invL[2];
 #pragma unroll
     for (int t = 0; t < T; ++t) {
-        const int64_t me = P.targets ? P.targets[gw * 32 + lane] : base + 32 * t + lane;
+        // Paired periodic walk: the lanes take the warp's 4x4x2 brick in rows along x, so that 4
+        // neighbouring lanes read neighbouring records of the correction table (x fastest)
+        const int ml32 = PKE ? (lane & 1) | ((lane >> 2) & 1) << 1 | (lane >> 4) << 2 | ((lane >> 1) & 1) << 3 | ((lane >> 3) & 1) << 4
+                             : lane;
+        const int64_t me = P.targets ? P.targets[gw * 32 + lane] : base + 32 * t + ml32;
         mcell[t] = me;
         if constexpr (PK) {   // the paired walk reads only the sibling-group copy of the cells
             const float* g = (const float*)(P.cell_soa + 8 * (me >> 3));
@@ -339,6 +512,10 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
     float2 k01 = make_float2(0.f, 0.f), k23 = k01, c01 = k01, c23 = k01;
     float2 nrx = make_float2(0.f, 0.f), nry = nrx, nrz = nrx;
     const float ith2 = PK ? (float)(1.0 / P.theta2) : 0.f;
+    // periodic axes: 1 / L and -L, 0 on isolated axes
+    const float2 ilx = make_float2(px ? (float)iLx : 0.f, px ? (float)iLx : 0.f), ily = make_float2(py ? (float)iLy : 0.f, py ? (float)iLy : 0.f),
+                 ilz = make_float2(pz ? (float)iLz : 0.f, pz ? (float)iLz : 0.f);
+    const float2 nlx = make_float2(-(float)Lx, -(float)Lx), nly = make_float2(-(float)Ly, -(float)Ly), nlz = make_float2(-(float)Lz, -(float)Lz);
     if constexpr (PK) {
         nrx = make_float2(-(float)rx[0], -(float)rx[0]);
         nry = make_float2(-(float)ry[0], -(float)ry[0]);
@@ -429,6 +606,29 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
                 const uint32_t sm = __ballot_sync(0xffffffffu, selfin);
                 n_int_w += 8u * lanes - (unsigned)__popc(sm & m0);
                 float2 sp = make_float2(0.f, 0.f), sax = sp, say = sp, saz = sp;
+                if constexpr (PKE) {
+                    // lanes outside the mask sit the group out: their lookups would only add L1 lines
+                    if (act[0]) {
+#pragma unroll 1
+                        for (int q = 0; q < 2; ++q) {
+                            const float4 X = __ldg(sx + q), Y = __ldg(sx + 2 + q);
+                            const float4 Z = __ldg(sx + 4 + q), M = __ldg(sx + 6 + q);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                const int j0 = 4 * q + 2 * h;
+                                float2 cx, cy, cz, m, dx, dy, dz, d2;
+                                pk_pair(X, Y, Z, M, h, cx, cy, cz, m);
+                                dx = pk_image(__fadd2_rn(cx, nrx), ilx, nlx);
+                                dy = pk_image(__fadd2_rn(cy, nry), ily, nly);
+                                dz = pk_image(__fadd2_rn(cz, nrz), ilz, nlz);
+                                d2 = pk_norm2(dx, dy, dz);
+                                ew_pair<EWM, POT, SUB>(P.ef, dx, dy, dz, d2, m, j0 != self0, j0 + 1 != self0, sp, sax);
+                            }
+                        }
+                        kahan_add2(k01, c01, sp);
+                        if constexpr (!POT) kahan_add2(k23, c23, sax);
+                    }
+                } else
                 // every lane sums all 8 cells (inactive lanes discard theirs below); only a group
                 // holding some lane's own cell needs the per-cell mask
                 if (sm == 0u) {
@@ -459,7 +659,7 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
                         }
                     }
                 }
-                if (act[0]) {
+                if (!PKE && act[0]) {
                     kahan_add2(k01, c01, make_float2(sp.x + sp.y, POT ? 0.f : sax.x + sax.y));
                     if constexpr (!POT) kahan_add2(k23, c23, make_float2(say.x + say.y, saz.x + saz.y));
                 }
@@ -561,11 +761,11 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
                 float2 sp = make_float2(0.f, 0.f), sax = sp, say = sp, saz = sp;
                 const bool a_act = act[0];
                 // BH: accept iff d^2 > h^2 / theta^2, the threshold formed once per pop
-                const float hb = a_act ? (float)h2 * ith2 : __int_as_float(0x7f800000);
+                const float hb = a_act ? (PKE ? P.thr[dep] : (float)h2 * ith2) : __int_as_float(0x7f800000);
                 const float2 hh = make_float2((float)h2, (float)h2);
                 const float2 gg = make_float2((float)G, (float)G), al = make_float2((float)alim[0], (float)alim[0]);
                 auto pairs = [&](unsigned ins) {
-#pragma unroll
+#pragma unroll(QUAD_UNROLL)
                     for (int q = 0; q < 2; ++q) {
                         const float4 X = __ldg(sx + q), Y = __ldg(sx + 2 + q);
                         const float4 Z = __ldg(sx + 4 + q), M = __ldg(sx + 6 + q);
@@ -575,7 +775,14 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
                             const int j0 = 4 * q + 2 * h;
                             float2 cx, cy, cz, m, dx, dy, dz, d2, inv;
                             pk_pair(X, Y, Z, M, h, cx, cy, cz, m);
-                            pk_sep(cx, cy, cz, nrx, nry, nrz, dx, dy, dz, d2);
+                            if constexpr (PKE) {
+                                dx = pk_image(__fadd2_rn(cx, nrx), ilx, nlx);
+                                dy = pk_image(__fadd2_rn(cy, nry), ily, nly);
+                                dz = pk_image(__fadd2_rn(cz, nrz), ilz, nlz);
+                                d2 = pk_norm2(dx, dy, dz);
+                            } else {
+                                pk_sep(cx, cy, cz, nrx, nry, nrz, dx, dy, dz, d2);
+                            }
                             bool mac0, mac1;
                             if constexpr (MAC == TS_MAC_MPE) {
                                 // eq. mpe, p = 1, as in the scalar path: G/d^2 (1 - b/d)^-2
@@ -606,7 +813,10 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
                             om[2 * h + 1] = __ballot_sync(0xffffffffu, a1);
                             // (no warp vote to skip pairs nobody accepts: most children are
                             // accepted, and the vote costs more than it saves)
-                            if constexpr (MAC == TS_MAC_MPE)
+                            if constexpr (PKE) {
+                                // (a lookup is worth a branch: lanes that accept neither child sit it out)
+                                if (a0 || a1) ew_pair<EWM, POT, SUB>(P.ef, dx, dy, dz, d2, m, a0, a1, sp, sax);
+                            } else if constexpr (MAC == TS_MAC_MPE)
                                 pk_interact_inv(dx, dy, dz, inv, m, a0, a1, sp, sax, say, saz);
                             else
                                 pk_interact_m<SUB>(dx, dy, dz, d2, m, a0, a1, sp, sax, say, saz);
@@ -615,8 +825,13 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
                             *(uint4*)&s_mask_w[TS_WALK_STACK - 8 + 4 * q][0] = make_uint4(om[0], om[1], om[2], om[3]);
                     }
                 };
-                if (sbd) pairs(box_bits(0)); else pairs(0u);
-                if (a_act) {
+                if constexpr (PKE) pairs(sbd ? box_bits(0) : 0u);   // (one copy of the lookups)
+                else if (sbd) pairs(box_bits(0));
+                else pairs(0u);
+                if (a_act && PKE) {
+                    kahan_add2(k01, c01, sp);
+                    if constexpr (!POT) kahan_add2(k23, c23, sax);
+                } else if (a_act) {
                     kahan_add2(k01, c01, make_float2(sp.x + sp.y, POT ? 0.f : sax.x + sax.y));
                     if constexpr (!POT) kahan_add2(k23, c23, make_float2(say.x + say.y, saz.x + saz.y));
                 }

@@ -3,18 +3,23 @@
 #pragma once
 #include "ts_walk_dev.cuh"
 
+
 // Walk kernel for one grid: one warp per 32 T target cells.  EWM: correction-table lookup
 // (0 trilinear, 1 Taylor, 2 run-time choice; see ewald_pair).
 // Resident CTAs per SM asked of the compiler: the paired isolated FP32 BH walk is held to 7 CTAs
 // (73 registers a thread), which measured 2.5 % faster than the compiler's own choice at the same
-// register count; the other instantiations keep the compiler's choice.
-template <typename R, int BCK, int MAC, int T>
+// register count.  The paired periodic walks wait for table records, so more resident warps help up to
+// where registers spill: Taylor 5 CTAs (96 registers; 64^3 disk 14.7 ms, 15.2 / 15.5 / 15.8 ms with 3,
+// 4, 6), trilinear 4 (64^3 box 3.55 ms, 3.72 / 3.58 / 4.27 ms with 3, 5, 6).  The other instantiations
+// keep the compiler's choice.
+template <typename R, int BCK, int MAC, int T, int EWM>
 struct WalkMinBlocks {
-    static constexpr int value = (sizeof(R) == 4 && BCK == 0 && MAC == TS_MAC_BH && T == 1) ? 7 : 1;
+    static constexpr bool paired = sizeof(R) == 4 && T == 1;
+    static constexpr int value = paired && BCK == 0 && MAC == TS_MAC_BH ? 7 : paired && BCK == 1 ? (EWM == 1 ? 5 : 4) : 1;
 };
 
 template <typename R, int BCK, int MAC, bool REL, int T, int EWM, bool POT = false, bool SUB = false>
-__global__ void __launch_bounds__(32 * TS_WALK_WARPS, (WalkMinBlocks<R, BCK, MAC, T>::value))
+__global__ void __launch_bounds__(32 * TS_WALK_WARPS, (WalkMinBlocks<R, BCK, MAC, T, EWM>::value))
     k_gravity_walk(const __grid_constant__ WalkParams P) {
     typedef typename RT<R>::V4 V4;
     __shared__ __align__(32) V4 s_com[TS_WALK_WARPS][8];
@@ -63,7 +68,7 @@ __global__ void __launch_bounds__(32 * TS_WALK_WARPS, (WalkMinBlocks<R, BCK, MAC
 template <typename R, int BCK, int MAC, bool REL, int T, int EWM = 2, bool POT = false, bool SUB = false>
 static cudaError_t launch_t(ts_ctx* c, const WalkParams& P) {
     // the paired walk of a mesh of extremely small cells keeps rsqrtf (see rsq)
-    if constexpr (sizeof(R) == 4 && BCK == 0 && T == 1 && !SUB)
+    if constexpr (sizeof(R) == 4 && BCK <= 1 && T == 1 && !SUB)
         if (P.tiny) return launch_t<R, BCK, MAC, REL, T, EWM, POT, true>(c, P);
     // warp lists: an upper bound
     const int64_t nwarps = P.targets ? P.ntargets / 32 : (P.leaf_end - P.leaf_begin) * (16 / T);
