@@ -150,6 +150,28 @@ cudaError_t make_walk_params(ts_ctx* c, const ts_gravity_params* p, void* pot, v
         if (p->mac == TS_MAC_BH)
             for (int d = 0; d <= TS_MAX_DEPTH; ++d) P.thr[d] = bh_threshold((float)P.theta2, c->geom.hmax2_32[d]);
     }
+    if (fp64 && bck == 0) {
+        // FP32 decisions of the FP64 walk.  A coordinate rounds by its magnitude times 2^-24 at most: S for
+        // a cell or box centre, S + d for a centre of mass at distance d (which lies outside the domain where
+        // masses have both signs).  An FP32 separation is then off by (2 S + 2 d) 2^-24 per axis, and d^2 by
+        // less than 4 sqrt(3) d (S + d) 2^-24 + 6 2^-24 d^2 + 12 S^2 2^-48 (arithmetic rounding included).  The
+        // band is twice that at the BH limit D = h / theta; nothing is decided in FP32 (thr = -1) where D^2
+        // leaves the FP32 range or the band would reach half of it.
+        double S = 0;
+        for (int a = 0; a < 3; ++a) S = std::max(S, std::max(fabs(c->dlo[a]), fabs(c->dlo[a] + c->L[a])));
+        const double u = ldexp(1.0, -24);
+        for (int d = 0; d <= TS_MAX_DEPTH; ++d) {
+            const double D2 = c->geom.hmax2_64[d] / P.theta2, D = sqrt(D2);
+            const double rel = 2 * (4 * sqrt(3.0) * S / D * u + 13 * u + 12 * S * S / D2 * u * u);
+            const bool ok = D2 > 1e-30 && D2 < 1e30 && rel < 0.5;   // (false for NaN)
+            P.thr[d] = ok ? (float)(D2 * (1 - rel)) : -1.f;
+            P.thr_hi[d] = ok ? (float)(D2 * (1 + rel)) : INFINITY;
+        }
+        // APE accepts at any distance: 4 sqrt(3) d S u <= t d^2 + (12 S^2 u^2) / t with t = 1e-5
+        P.ape_s0 = (float)(2 * (12 * S * S * u * u / 1e-5 + 12 * S * S * u * u));
+        P.box_tol = S < 1e30 ? (float)(8 * S * u) : INFINITY;
+        P.ncen32 = c->d_ncen32;
+    }
     P.pot = pot;
     P.acc = acc;
     P.status = c->d_status;

@@ -72,7 +72,11 @@ struct WalkParams {
     unsigned long long* blk_counts;   // nullable: interactions per leaf-block (warp-list and full walks)
     EwaldDev ew;
     EwF32 ef;
-    float thr[TS_MAX_DEPTH + 1];      // paired periodic BH walk: accept iff d^2 > thr[depth]
+    // paired periodic BH walk: accept iff d^2 > thr[depth]; FP64 walk: FP32 d^2 <= thr[depth] is rejected
+    // and > thr_hi[depth] accepted for certain (BH), and the FP32 errors of d^2 (APE) and of the box test
+    float thr[TS_MAX_DEPTH + 1], thr_hi[TS_MAX_DEPTH + 1];
+    float ape_s0, box_tol;
+    const float4* ncen32;
     void* pot;
     void* acc;
     int* status;

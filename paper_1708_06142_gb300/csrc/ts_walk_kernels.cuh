@@ -91,7 +91,9 @@ template <typename R, int BCK, int MAC, bool REL>
 static cudaError_t dispatch_t(ts_ctx* c, const WalkParams& P, int T) {
     if (T == 4) return launch_t<R, BCK, MAC, REL, 4>(c, P);
     if (T == 2) return launch_t<R, BCK, MAC, REL, 2>(c, P);
-    if constexpr (BCK == 1)
+    if constexpr (sizeof(R) == 8 && BCK == 0)
+        return cudaErrorInvalidValue;   // (ts_walk64.cuh)
+    else if constexpr (BCK == 1)
         return P.ew.taylor ? launch_t<R, BCK, MAC, REL, 1, 1>(c, P) : launch_t<R, BCK, MAC, REL, 1, 0>(c, P);
     else
         return launch_t<R, BCK, MAC, REL, 1>(c, P);
