@@ -781,11 +781,12 @@ ts_status ensure_noderay(ts_ctx* c, int nside, const int dims[3], double pmin, d
     std::vector<double> dense(nent * npix);
     TS_CUDA(cudaMemcpyAsync(dense.data(), c->d_nr_dense, sizeof(double) * dense.size(), cudaMemcpyDeviceToHost, c->stream));
     TS_CUDA(cudaStreamSynchronize(c->stream));
-    // one 16-byte record of up to 4 (sub-cube count << 8 | pixel) pairs per entry; the weights are
-    // counts over nsub^3 (the table kernel counts sub-cube centres per pixel), so counts are exact;
-    // a longer row keeps 3 pairs and (offset << 8 | 255) into the continuation array
+    // one 32-byte record per entry: the sub-cube counts of up to 4 pixels (FP32), their map offsets
+    // (pixel * 32 lanes * 4 bytes) in 16-bit halves, and 0 or the index of the record that continues the
+    // row.  The weights are counts over nsub^3 (the table kernel counts sub-cube centres per pixel), so
+    // counts are exact; an unused slot has count 0 at a pixel that the record does not name otherwise.
     const double n3 = (double)nsub * nsub * nsub;
-    std::vector<uint32_t> rec(nent * 4, 0u), more;
+    std::vector<uint32_t> rec(nent * 8, 0u), more(8, 0u);   // (record 0 of the continuations is unused)
     std::vector<uint32_t> row;
     for (size_t e = 0; e < nent; ++e) {
         row.clear();
@@ -799,19 +800,37 @@ ts_status ensure_noderay(ts_ctx* c, int nside, const int dims[3], double pmin, d
             }
         }
         if (row.empty()) return ts_fail(TS_ERR_NUMERIC, "node-ray table: an entry with no pixel");
-        if (row.size() <= 4) {
-            for (size_t k = 0; k < row.size(); ++k) rec[4 * e + k] = row[k];
-        } else {
-            for (int k = 0; k < 3; ++k) rec[4 * e + k] = row[k];
-            if (more.size() >= (1u << 24)) return ts_fail(TS_ERR_UNSUPPORTED, "node-ray table: rows too long");
-            rec[4 * e + 3] = ((uint32_t)more.size() << 8) | 255u;
-            more.push_back((uint32_t)(row.size() - 3));
-            more.insert(more.end(), row.begin() + 3, row.end());
+        auto put = [&](uint32_t* r, size_t k0) {   // pixels k0 .. k0 + 3 of the row
+            uint32_t pix[4], free = 0;
+            for (uint32_t k = 0; k < 4; ++k) {
+                const bool have = k0 + k < row.size();
+                const float w = have ? (float)(row[k0 + k] >> 8) : 0.f;
+                if (have) {
+                    pix[k] = row[k0 + k] & 255u;
+                } else {   // (npix >= 12, so a pixel is left)
+                    while (std::find(pix, pix + k, free) != pix + k) ++free;
+                    pix[k] = free;
+                }
+                memcpy(&r[k], &w, 4);
+            }
+            r[4] = pix[0] * 128u | (pix[1] * 128u) << 16;
+            r[5] = pix[2] * 128u | (pix[3] * 128u) << 16;
+        };
+        const size_t it = e / (dims[1] * dims[2]), ip = e / dims[2] % dims[1], is = e % dims[2];
+        const size_t re = (is * dims[0] + it) * dims[1] + ip;   // psi slowest, phi fastest
+        put(&rec[8 * re], 0);
+        uint32_t* link = &rec[8 * re + 6];
+        for (size_t k0 = 4; k0 < row.size(); k0 += 4) {
+            const size_t at = more.size();
+            if (at >= (1u << 27)) return ts_fail(TS_ERR_UNSUPPORTED, "node-ray table: rows too long");
+            *link = (uint32_t)(at / 8);
+            more.resize(at + 8, 0u);
+            put(&more[at], k0);
+            link = &more[at + 6];
         }
     }
-    if (more.empty()) more.push_back(0u);
-    TS_CUDA(dalloc(c->d_nr_rec, nent));
-    TS_CUDA(dalloc(c->d_nr_more, more.size()));
+    TS_CUDA(dalloc(c->d_nr_rec, 2 * nent));
+    TS_CUDA(dalloc(c->d_nr_more, more.size() / 4));
     TS_CUDA(cudaMemcpyAsync(c->d_nr_rec, rec.data(), sizeof(uint32_t) * rec.size(), cudaMemcpyHostToDevice, c->stream));
     TS_CUDA(cudaMemcpyAsync(c->d_nr_more, more.data(), sizeof(uint32_t) * more.size(), cudaMemcpyHostToDevice,
                             c->stream));

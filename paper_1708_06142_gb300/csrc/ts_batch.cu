@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(32 * TS_WALK_WARPS) k_batch_walk(const __grid_
                 __syncwarp();
             }
             if constexpr (CLS == 2)
-                col_walk_warp(W.cp, local, lane, map, W.com, W.cen, W.cstack, W.half, W.h2);
+                col_walk_warp<0, SUB>(W.cp, local, lane, map, W.com, W.cen, W.cstack, W.half, W.h2);
             else
                 walk_warp<float, CLS, MAC, false, 1, EWM, false, SUB>(W.wp, local, warp, lane, W.com, W.cen, W.cw, W.mask,
                                                                       W.half, W.h2, nullptr);
@@ -260,9 +260,9 @@ static int periodic_kind(const int bc[3]) {
 template <int MAC, int CLS, int EWM = 2, bool SUB = false>
 static cudaError_t launch_cls(ts_batch* b, const BatchArgs& A, cudaStream_t st) {
     // a batch holding a mesh of extremely small cells keeps rsqrtf (see rsq)
-    if constexpr (CLS <= 1 && !SUB)
+    if constexpr (!SUB)
         for (size_t i = 0; i < b->ctx.size(); ++i)
-            if (b->h_wp[i].tiny) return launch_cls<MAC, CLS, EWM, true>(b, A, st);
+            if (CLS == 2 ? b->h_cp[i].tiny : b->h_wp[i].tiny) return launch_cls<MAC, CLS, EWM, true>(b, A, st);
     const size_t smem = TS_WALK_WARPS * batch_warp_smem(A.npix);
     cudaError_t e = cudaFuncSetAttribute(k_batch_walk<MAC, CLS, EWM, SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -497,7 +497,8 @@ extern "C" ts_status ts_batch_run(ts_batch* b, const ts_gravity_params* gp, void
                                  (uint64_t)(density != nullptr)};
     sig.push_back((uint64_t)b->mode);
     sig.push_back((uint64_t)b->nstreams);
-    for (int i = 0; i < n; ++i) sig.push_back((uint64_t)b->h_wp[i].tiny);   // chooses the kernel
+    for (int i = 0; i < n; ++i)   // (they choose kernels)
+        sig.push_back((uint64_t)((gp ? b->h_wp[i].tiny : 0) | (cp ? b->h_cp[i].tiny : 0)));
     for (int i = 0; i < n; ++i) {
         sig.push_back(density ? (uint64_t)density[i] : 0);
         sig.push_back(gp ? (uint64_t)pot[i] : 0);

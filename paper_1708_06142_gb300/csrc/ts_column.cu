@@ -13,7 +13,7 @@
 // the target to the node.  Each lane's map lives in shared memory as [pixel][lane] (conflict-free
 // scatter).  The own cell adds rho dx / 2 to every pixel.
 //
-// Roofline: the scatter is FP32/shared-memory bound; the output ([ncell][N_PIX] floats, 403 MB for
+// Roofline: bound by instruction issue and the L1 data path (node-ray records and map updates); the output ([ncell][N_PIX] floats, 403 MB for
 // 128^3 cells at N_PIX = 48) is an HBM write.
 #include <math.h>
 #include <string.h>
@@ -87,8 +87,8 @@ cudaError_t launch_noderay_dense(ts_ctx* c, int nside, const int dims[3], double
 
 #include "ts_column_dev.cuh"
 
-template <int NQ>
-__global__ void __launch_bounds__(32 * TS_WALK_WARPS) k_column_walk(const __grid_constant__ ColParams P) {
+template <int NQ, bool SUB>
+__global__ void __launch_bounds__(32 * TS_WALK_WARPS, ColTune<NQ>::min_ctas) k_column_walk(const __grid_constant__ ColParams P) {
     extern __shared__ float s_map[];   // [TS_WALK_WARPS][1 + NQ][npix][32]
     __shared__ __align__(16) float4 s_com[TS_WALK_WARPS][8];
     __shared__ __align__(16) float4 s_cen[TS_WALK_WARPS][8];
@@ -104,29 +104,28 @@ __global__ void __launch_bounds__(32 * TS_WALK_WARPS) k_column_walk(const __grid
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t gw = (int64_t)blockIdx.x * TS_WALK_WARPS + warp;
     if (gw * 32 >= P.ncell) return;
-    col_walk_warp<NQ>(P, gw, lane, s_map + (size_t)warp * (1 + NQ) * P.npix * 32, s_com[warp], s_cen[warp],
+    col_walk_warp<NQ, SUB>(P, gw, lane, s_map + (size_t)warp * (1 + NQ) * P.npix * 32, s_com[warp], s_cen[warp],
                       s_stack[warp], s_half, s_h2, s_q[warp]);
 }
 
 static size_t col_smem(const ColParams& P, int nq) { return sizeof(float) * (size_t)(1 + nq) * P.npix * 32 * TS_WALK_WARPS; }
 
-static cudaError_t col_launch(ts_ctx* c, const ColParams& P, int nq) {
-    const size_t smem = col_smem(P, nq);
+template <int NQ, bool SUB>
+static cudaError_t col_launch_t(ts_ctx* c, const ColParams& P) {
+    // meshes of extremely small cells keep the functions that take subnormal arguments (see rsq)
+    if constexpr (!SUB)
+        if (P.tiny) return col_launch_t<NQ, true>(c, P);
+    const size_t smem = col_smem(P, NQ);
     const int64_t nwarps = c->ncell / 32;
     const int grid = (int)((nwarps + TS_WALK_WARPS - 1) / TS_WALK_WARPS);
-    cudaError_t e = cudaSuccess;
-    if (nq == 0) {
-        e = cudaFuncSetAttribute(k_column_walk<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) k_column_walk<0><<<grid, 32 * TS_WALK_WARPS, smem, c->stream>>>(P);
-    } else if (nq == 1) {
-        e = cudaFuncSetAttribute(k_column_walk<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) k_column_walk<1><<<grid, 32 * TS_WALK_WARPS, smem, c->stream>>>(P);
-    } else {
-        e = cudaFuncSetAttribute(k_column_walk<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) k_column_walk<2><<<grid, 32 * TS_WALK_WARPS, smem, c->stream>>>(P);
-    }
+    cudaError_t e = cudaFuncSetAttribute(k_column_walk<NQ, SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
+    k_column_walk<NQ, SUB><<<grid, 32 * TS_WALK_WARPS, smem, c->stream>>>(P);
     return cudaGetLastError();
+}
+
+static cudaError_t col_launch(ts_ctx* c, const ColParams& P, int nq) {
+    return nq == 0 ? col_launch_t<0, false>(c, P) : nq == 1 ? col_launch_t<1, false>(c, P) : col_launch_t<2, false>(c, P);
 }
 
 // Kernel parameters of one context's column walk; the node-ray table comes from `tab` (a context
@@ -146,12 +145,19 @@ cudaError_t make_col_params(ts_ctx* c, const ts_ctx* tab, const ts_column_params
     P.ncell = c->ncell;
     P.theta2 = (float)(p->theta * p->theta);
     P.eta = (float)p->safe_box;
-    P.max_dist2 = p->max_dist > 0 ? (float)(p->max_dist * p->max_dist) : 0.f;
+    P.max_dist2 = p->max_dist > 0 ? (float)(p->max_dist * p->max_dist) : INFINITY;
+    if (!(P.max_dist2 > 0.f)) P.max_dist2 = INFINITY;   // (a square that underflows: unlimited)
     P.geom = c->d_geom;
     P.npix = tab->nr_dims[3];
-    P.nth = tab->nr_dims[0];
+    P.nthf = (float)tab->nr_dims[0];
+    P.nth1 = (float)(tab->nr_dims[0] - 1);
+    P.nphf = (float)tab->nr_dims[1];
+    P.nph1 = (float)(tab->nr_dims[1] - 1);
+    P.nps1 = (float)(tab->nr_dims[2] - 1);
+    P.tiny = c->min_edge < 1e-11 ? 1 : 0;   // (as for the gravity walk)
+    for (int d = 0; d <= TS_MAX_DEPTH; ++d) P.thr[d] = bh_threshold(P.theta2, c->geom.hmax2_32[d]);
     P.nph = tab->nr_dims[1];
-    P.nps = tab->nr_dims[2];
+    P.nth = tab->nr_dims[0];
     P.psi_lmin = (float)log2(tab->nr_psi[0]);
     P.psi_lscale = (float)(tab->nr_dims[2] / log2(tab->nr_psi[1] / tab->nr_psi[0]));
     // safe-box test only at depths where a target inside the box could pass the BH MAC (the same
@@ -165,7 +171,8 @@ cudaError_t make_col_params(ts_ctx* c, const ts_ctx* tab, const ts_column_params
     // the pairs store sub-cube counts: their weight is count / nsub^3, folded into 1 / Omega_pix
     P.inv_omega = (float)(P.npix / (4.0 * M_PI) / ((double)tab->nr_nsub * tab->nr_nsub * tab->nr_nsub));
     P.leaf_size = c->d_leaf_size;
-    P.nr_rec = tab->d_nr_rec;
+    const uint32_t bias = 0x4b000000u * (uint32_t)(P.nth * P.nph + P.nph + 1);
+    P.nr_rec = (const float4*)((uintptr_t)tab->d_nr_rec - (uintptr_t)bias * 32u);
     P.nr_more = tab->d_nr_more;
     P.out = cols;
     P.status = c->d_status;

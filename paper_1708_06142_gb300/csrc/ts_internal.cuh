@@ -160,8 +160,8 @@ struct ts_ctx {
     int nr_nside = 0, nr_dims[4] = {0, 0, 0, 0}, nr_nsub = 0, nr_kmax = 0;   // nr_kmax: pairs in all
     double nr_psi[2] = {0, 0};
     double* d_nr_dense = nullptr;    // FP64 [ntheta][nphi][npsi][npix]
-    uint4* d_nr_rec = nullptr;       // [entry] up to 4 (sub-cube count << 8) | pixel pairs (npix <= 192)
-    uint32_t* d_nr_more = nullptr;   // continuation of the rows longer than 4 pairs
+    float4* d_nr_rec = nullptr;      // [entry][2] 32-byte records of up to 4 pixels (see ColHit; npix <= 192)
+    float4* d_nr_more = nullptr;     // records of the pixels beyond the first 4 of a row
 
     // learned Ewald-correction surrogate (2P1I)
     bool have_mlp = false;
@@ -237,6 +237,7 @@ ts_status ensure_bmoments(ts_ctx* c, bool fp64);
 cudaError_t launch_gravity_walk(ts_ctx* c, const ts_gravity_params* p, void* pot, void* acc);
 ts_status validate_gravity(ts_ctx* c, const ts_gravity_params* p);
 int ew_kind(const int bc[3]);
+float bh_threshold(float theta2, float h2);
 cudaError_t launch_zero_mean(ts_ctx* c, int precision, void* pot);
 cudaError_t launch_num_diff(ts_ctx* c, int precision, const void* pot, void* acc);
 ts_status ensure_numdiff(ts_ctx* c);

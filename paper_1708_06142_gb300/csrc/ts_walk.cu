@@ -53,7 +53,7 @@ static cudaError_t upload_geom(ts_ctx* c, WalkGeom** out) {
 
 // The largest x with !(h2 < theta2 x) in FP32: the scalar form of the BH test, h2 < theta2 d^2, as one
 // comparison d^2 > x with the same decision for every d^2 (the product is monotonic in x).
-static float bh_threshold(float theta2, float h2) {
+float bh_threshold(float theta2, float h2) {
     uint32_t lo = 0, hi = 0x7f800000u;   // +0 .. +inf: the bits order like the values
     while (lo < hi) {
         const uint32_t mid = lo + (hi - lo + 1) / 2;

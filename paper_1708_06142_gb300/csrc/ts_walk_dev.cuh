@@ -10,6 +10,7 @@
 
 #include "ts_internal.cuh"
 #include "ts_mlp.cuh"
+#include "ts_pair.cuh"
 
 // Per-warp row buffers of the learned-correction mode (one pop: up to 8 children x 32 lanes).
 #define MLP_ROWS 256
@@ -91,17 +92,6 @@ __device__ __forceinline__ float rint_t(float x) { return rintf(x); }
 __device__ __forceinline__ double rint_t(double x) { return rint(x); }
 __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
-// 1/sqrt(x).  SUB = false: the hardware instruction alone, which flushes subnormal inputs.  rsqrtf
-// also rescales those, three more instructions on every call (24 of the ~200 of a popped group: the
-// 2M-cell Plummer BH walk ran 9 % longer with it); it is kept for meshes whose cells are so small
-// that a squared separation can be subnormal (WalkParams::tiny).  Normal inputs give the same bits.
-template <bool SUB>
-__device__ __forceinline__ float rsq(float x) {
-    if constexpr (SUB) return rsqrtf(x);
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 __device__ __forceinline__ float log_t(float x) { return logf(x); }
 __device__ __forceinline__ double log_t(double x) { return log(x); }
 
@@ -288,15 +278,6 @@ __device__ __forceinline__ void ewald_pair(const EwaldDev& E, R dx, R dy, R dz, 
     Az = dz * inv3 + (dz < (R)0 ? -cz : cz);
 }
 
-// 32-byte record by one 256-bit load.  Measured on GB300 with scattered addresses: a 128-bit load
-// costs the L1 one cycle per distinct 128-byte line of the warp, a 256-bit load half a cycle per
-// distinct line of each group of 4 lanes, so a record costs half or less of two 128-bit loads.
-__device__ __forceinline__ void ld_rec(const float4* p, float4& a, float4& b) {
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
-        : "l"(p));
-}
-
 // t with its sign flipped where d is negative (A_c is odd in its own axis)
 __device__ __forceinline__ float flip(float t, float d) {
     return __uint_as_float(__float_as_uint(t) ^ (__float_as_uint(d) & 0x80000000u));
@@ -304,22 +285,6 @@ __device__ __forceinline__ float flip(float t, float d) {
 
 __device__ __forceinline__ float2 lerp2(float2 a, float2 b, float2 f) {
     return __ffma2_rn(f, __ffma2_rn(a, make_float2(-1.f, -1.f), b), a);
-}
-
-// Minimum image of two separations at once: d - L rint(d / L), the rounding to the nearest integer by
-// adding and subtracting 1.5 * 2^23 (exact below 2^22; two packed additions where rintf needs the
-// conversion unit for each value).  An isolated axis has 1 / L = L = 0.
-__device__ __forceinline__ float2 pk_image(float2 d, float2 iL, float2 nL) {
-    const float2 M = make_float2(12582912.f, 12582912.f), N = make_float2(-12582912.f, -12582912.f);
-    return __ffma2_rn(__fadd2_rn(__fadd2_rn(__fmul2_rn(d, iL), M), N), nL, d);
-}
-
-// d^2 as the scalar kernels form it, fma(dx, dx, dy dy) + dz dz with the last product rounded by
-// itself, so that every MAC decision is theirs bit for bit.  (The last addition is scalar: a packed
-// one is fused with the packed product.)
-__device__ __forceinline__ float2 pk_norm2(float2 dx, float2 dy, float2 dz) {
-    const float2 a = __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)), b = __fmul2_rn(dz, dz);
-    return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
 }
 
 // The paired periodic walk's lookup of a pair of children of which this lane accepts acc[0] and/or
