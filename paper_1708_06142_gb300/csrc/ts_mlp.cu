@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(128) k_mlp_eval(const void* __restrict__ img, 
         }
         __syncwarp();
         const int nrows = n - m0 < 16 ? (int)(n - m0) : 16;
-        mlp_eval_tile(M, s_feat[warp], s_out[warp], 0, nrows, lane);
+        mlp_eval_tile<1>(M, s_feat[warp], s_out[warp], 0, nrows, lane);
         __syncwarp();
         if (lane < nrows) ((float4*)out)[m0 + lane] = s_out[warp][lane];
         __syncwarp();

@@ -45,7 +45,7 @@ __device__ __forceinline__ MlpView mlp_view(const void* base) {
 }
 
 __device__ __forceinline__ void mma_bf16_16816(float c[4], const uint32_t a[4], const uint32_t b[2]) {
-    asm volatile(
+    asm(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
         "{%0,%1,%2,%3};\n"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
@@ -62,8 +62,6 @@ __device__ __forceinline__ float tanh_fast(float x) {
     asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-
-__device__ __forceinline__ float silu_f(float z) { return 0.5f * z * (1.0f + tanh_fast(0.5f * z)); }
 
 // d silu / dz = s (1 + z (1 - s)), s = sigmoid(z) = (1 + tanh(z/2)) / 2
 __device__ __forceinline__ float silu_grad_f(float z) {
@@ -107,93 +105,119 @@ __device__ __forceinline__ uint4 mlp_feat_pack(float f0, float f1, float f2, flo
     return r;
 }
 
-// Network output for 16 rows m0 .. m0+15 whose features are feat[row] (mlp_feat_pack: 8 bf16).
-// out[row] receives the de-normalised (C, A_cx, A_cy, A_cz) for rows < nrows.
+// silu(z) = z/2 (1 + tanh(z/2)) of two values, as a BF16 pair
+__device__ __forceinline__ uint32_t silu_pack(float z0, float z1) {
+    const float2 h = __fmul2_rn(make_float2(z0, z1), make_float2(0.5f, 0.5f));
+    const float2 r = __fmul2_rn(h, __fadd2_rn(make_float2(tanh_fast(h.x), tanh_fast(h.y)), make_float2(1.f, 1.f)));
+    return pack_bf16(r.x, r.y);
+}
+
+// Network output for 16 MT rows m0 .. m0 + 16 MT - 1 whose features are feat[row] (mlp_feat_pack: 8 bf16).
+// out[row] receives the de-normalised (C, A_cx, A_cy, A_cz) for rows < nrows.  The MT row tiles share every
+// weight fragment, and the k-steps are the outer loop, so that 8 MT independent MMAs follow one another: the
+// walk is bound by the latency of these chains (tensor pipe 43 % busy with MT = 2).  32^3 disk: 19.2 ms with
+// one tile and the k-steps innermost, 18.1 / 17.1 / 18.4 ms with MT = 1 / 2 / 3.
+template <int MT>
 __device__ __forceinline__ void mlp_eval_tile(const MlpView& M, const uint4* feat, float4* out, int m0, int nrows,
                                               int lane) {
     const int g = lane >> 2, t = lane & 3;
-    uint32_t a[4];
-    {   // columns 2t, 2t + 1 of rows g and g + 8: word t of the packed row
-        const uint4 f0 = feat[m0 + g], f1 = feat[m0 + g + 8];
-        a[0] = t == 0 ? f0.x : t == 1 ? f0.y : t == 2 ? f0.z : f0.w;
-        a[1] = t == 0 ? f1.x : t == 1 ? f1.y : t == 2 ? f1.z : f1.w;
-    }
-    a[2] = 0u;
-    a[3] = 0u;
-    uint32_t h[4][4];
+    uint32_t h[MT][4][4];
     {   // layer 1: K = 16 (4 real), N = 64
-        float z[8][4];
+        uint32_t a[MT][4];
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {   // columns 2t, 2t + 1 of rows g and g + 8: word t of the packed row
+            const uint32_t* f = (const uint32_t*)(feat + m0 + 16 * m);
+            a[m][0] = f[4 * g + t];
+            a[m][1] = f[4 * (g + 8) + t];
+            a[m][2] = a[m][3] = 0u;
+        }
+        float z[MT][8][4];
 #pragma unroll
         for (int nt = 0; nt < 8; nt += 2) {
             uint32_t b[4];
             bfrag_ldsm(b, M.w + MLP_OFF_W1, MLP_LD1, nt * 8, 0, 8, 0, lane);   // n-tiles nt, nt + 1
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-                const float b0 = M.f[(nt + u) * 8 + 2 * t], b1 = M.f[(nt + u) * 8 + 2 * t + 1];
-                z[nt + u][0] = b0; z[nt + u][1] = b1; z[nt + u][2] = b0; z[nt + u][3] = b1;
-                mma_bf16_16816(z[nt + u], a, b + 2 * u);
+                const float2 bb = *(const float2*)(M.f + (nt + u) * 8 + 2 * t);
+#pragma unroll
+                for (int m = 0; m < MT; ++m) {
+                    z[m][nt + u][0] = z[m][nt + u][2] = bb.x;
+                    z[m][nt + u][1] = z[m][nt + u][3] = bb.y;
+                    mma_bf16_16816(z[m][nt + u], a[m], b + 2 * u);
+                }
             }
         }
 #pragma unroll
-        for (int kt = 0; kt < 4; ++kt) {
-            h[kt][0] = pack_bf16(silu_f(z[2 * kt][0]), silu_f(z[2 * kt][1]));
-            h[kt][1] = pack_bf16(silu_f(z[2 * kt][2]), silu_f(z[2 * kt][3]));
-            h[kt][2] = pack_bf16(silu_f(z[2 * kt + 1][0]), silu_f(z[2 * kt + 1][1]));
-            h[kt][3] = pack_bf16(silu_f(z[2 * kt + 1][2]), silu_f(z[2 * kt + 1][3]));
-        }
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int kt = 0; kt < 4; ++kt) {
+                h[m][kt][0] = silu_pack(z[m][2 * kt][0], z[m][2 * kt][1]);
+                h[m][kt][1] = silu_pack(z[m][2 * kt][2], z[m][2 * kt][3]);
+                h[m][kt][2] = silu_pack(z[m][2 * kt + 1][0], z[m][2 * kt + 1][1]);
+                h[m][kt][3] = silu_pack(z[m][2 * kt + 1][2], z[m][2 * kt + 1][3]);
+            }
     }
 #pragma unroll
     for (int layer = 0; layer < 2; ++layer) {   // layers 2 and 3: K = N = 64
         const __nv_bfloat16* W = M.w + (layer == 0 ? MLP_OFF_W2 : MLP_OFF_W3);
         const float* bias = M.f + 64 * (layer + 1);
-        float z[8][4];
+        float z[MT][8][4];
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
-            const float b0 = bias[nt * 8 + 2 * t], b1 = bias[nt * 8 + 2 * t + 1];
-            z[nt][0] = b0; z[nt][1] = b1; z[nt][2] = b0; z[nt][3] = b1;
-        }
+            const float2 bb = *(const float2*)(bias + nt * 8 + 2 * t);
 #pragma unroll
-        for (int nt = 0; nt < 8; nt += 2) {
-#pragma unroll
-            for (int kt = 0; kt < 4; ++kt) {
-                uint32_t b[4];
-                bfrag_ldsm(b, W, MLP_LD, nt * 8, kt * 16, 8, 0, lane);   // n-tiles nt, nt + 1
-                mma_bf16_16816(z[nt], h[kt], b);
-                mma_bf16_16816(z[nt + 1], h[kt], b + 2);
+            for (int m = 0; m < MT; ++m) {
+                z[m][nt][0] = z[m][nt][2] = bb.x;
+                z[m][nt][1] = z[m][nt][3] = bb.y;
             }
         }
 #pragma unroll
         for (int kt = 0; kt < 4; ++kt) {
-            h[kt][0] = pack_bf16(silu_f(z[2 * kt][0]), silu_f(z[2 * kt][1]));
-            h[kt][1] = pack_bf16(silu_f(z[2 * kt][2]), silu_f(z[2 * kt][3]));
-            h[kt][2] = pack_bf16(silu_f(z[2 * kt + 1][0]), silu_f(z[2 * kt + 1][1]));
-            h[kt][3] = pack_bf16(silu_f(z[2 * kt + 1][2]), silu_f(z[2 * kt + 1][3]));
+#pragma unroll
+            for (int nt = 0; nt < 8; nt += 2) {
+                uint32_t b[4];
+                bfrag_ldsm(b, W, MLP_LD, nt * 8, kt * 16, 8, 0, lane);   // n-tiles nt, nt + 1
+#pragma unroll
+                for (int m = 0; m < MT; ++m) {
+                    mma_bf16_16816(z[m][nt], h[m][kt], b);
+                    mma_bf16_16816(z[m][nt + 1], h[m][kt], b + 2);
+                }
+            }
         }
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int kt = 0; kt < 4; ++kt) {
+                h[m][kt][0] = silu_pack(z[m][2 * kt][0], z[m][2 * kt][1]);
+                h[m][kt][1] = silu_pack(z[m][2 * kt][2], z[m][2 * kt][3]);
+                h[m][kt][2] = silu_pack(z[m][2 * kt + 1][0], z[m][2 * kt + 1][1]);
+                h[m][kt][3] = silu_pack(z[m][2 * kt + 1][2], z[m][2 * kt + 1][3]);
+            }
     }
     // layer 4: N = 8 (4 real outputs), K = 64
-    const float* b4 = M.f + 192;
-    float z[4] = {b4[2 * t], b4[2 * t + 1], b4[2 * t], b4[2 * t + 1]};
+    float z[MT][4];
+    {
+        const float2 bb = *(const float2*)(M.f + 192 + 2 * t);
+#pragma unroll
+        for (int m = 0; m < MT; ++m) { z[m][0] = z[m][2] = bb.x; z[m][1] = z[m][3] = bb.y; }
+    }
 #pragma unroll
     for (int kt = 0; kt < 4; kt += 2) {
         uint32_t b[4];
         bfrag_ldsm(b, M.w + MLP_OFF_W4, MLP_LD, 0, kt * 16, 0, 16, lane);   // k-tiles kt, kt + 1
-        mma_bf16_16816(z, h[kt], b);
-        mma_bf16_16816(z, h[kt + 1], b + 2);
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+            mma_bf16_16816(z[m], h[m][kt], b);
+            mma_bf16_16816(z[m], h[m][kt + 1], b + 2);
+        }
     }
     if (t < 2) {
-        const float* sc = M.f + 200;
-        const float* of = M.f + 204;
-        const int c0 = 2 * t;
-        const int r0 = m0 + g, r1 = m0 + g + 8;
-        if (r0 < nrows) {
-            float* o = (float*)&out[r0];
-            o[c0] = z[0] * sc[c0] + of[c0];
-            o[c0 + 1] = z[1] * sc[c0 + 1] + of[c0 + 1];
-        }
-        if (r1 < nrows) {
-            float* o = (float*)&out[r1];
-            o[c0] = z[2] * sc[c0] + of[c0];
-            o[c0 + 1] = z[3] * sc[c0 + 1] + of[c0 + 1];
+        const float2 sc = *(const float2*)(M.f + 200 + 2 * t), of = *(const float2*)(M.f + 204 + 2 * t);
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+            const int r0 = m0 + 16 * m + g, r1 = r0 + 8;
+            if (r0 < nrows) *(float2*)((float*)&out[r0] + 2 * t) = make_float2(z[m][0] * sc.x + of.x, z[m][1] * sc.y + of.y);
+            if (r1 < nrows) *(float2*)((float*)&out[r1] + 2 * t) = make_float2(z[m][2] * sc.x + of.x, z[m][3] * sc.y + of.y);
         }
     }
 }
