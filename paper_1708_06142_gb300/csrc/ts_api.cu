@@ -371,7 +371,8 @@ static ts_status ingest_mesh(ts_ctx* c, const ts_mesh* m) {
     chk(dalloc(c->d_leaf_nid, nleaf));
     chk(dalloc(c->d_leaf_lo, 3 * (size_t)nleaf));
     chk(dalloc(c->d_leaf_size, 3 * (size_t)nleaf));
-    chk(dalloc(c->d_amr_order, c->amr_order.size() + c->amr_level_off.size()));
+    const size_t ngrp = (size_t)(nb - 1) / 8;   // sibling groups of amr nodes
+    chk(dalloc(c->d_amr_order, c->amr_order.size() + c->amr_level_off.size() + 2 * ngrp));
     chk(dalloc(c->d_ncom32, nint));
     chk(dalloc(c->d_ncen32, nint));
     chk(dalloc(c->d_ncom64, nint));
@@ -384,9 +385,15 @@ static ts_status ingest_mesh(ts_ctx* c, const ts_mesh* m) {
     chk(cudaMemcpyAsync(c->d_leaf_nid, leaf_nid.data(), sizeof(int) * nleaf, cudaMemcpyHostToDevice, c->stream));
     chk(cudaMemcpyAsync(c->d_leaf_lo, leaf_lo.data(), sizeof(double) * 3 * nleaf, cudaMemcpyHostToDevice, c->stream));
     chk(cudaMemcpyAsync(c->d_leaf_size, leaf_size.data(), sizeof(double) * 3 * nleaf, cudaMemcpyHostToDevice, c->stream));
-    {   // node ids of the non-leaf blocks, then the per-round offsets
+    {   // node ids of the non-leaf blocks, the per-round offsets, the groups' parents and counts
         std::vector<int> ord(c->amr_order);
         ord.insert(ord.end(), c->amr_level_off.begin(), c->amr_level_off.end());
+        c->d_amr_parent = c->d_amr_order + ord.size();
+        c->d_amr_count = c->d_amr_parent + ngrp;
+        const size_t at = ord.size();
+        ord.resize(at + 2 * ngrp, 0);
+        for (int b = 0; b < nb; ++b)
+            if (m->child[8 * b] >= 0) ord[at + (size_t)(c->blk_nid[m->child[8 * b]] - 1) / 8] = c->blk_nid[b];
         chk(cudaMemcpyAsync(c->d_amr_order, ord.data(), sizeof(int) * ord.size(), cudaMemcpyHostToDevice, c->stream));
         chk(cudaStreamSynchronize(c->stream));
     }

@@ -1,14 +1,17 @@
-// Tree build (Sec. 2.1): cell masses and bottom-up FP64 node moments.
+// Tree build (Sec. 2.1): cell masses and bottom-up FP64 node moments, one kernel.
 //
 // k_blocktree: one CTA of 512 threads per leaf-block.  Each thread reads one density value
 // (coalesced, natural cell order), forms m = rho dV and the cell centre in FP64, and stores them
 // in shared memory at the cell's Morton slot.  The 64 level-2 nodes, 8 level-1 nodes and the
-// leaf-block node are then summed in shared memory, children in octant order.  Products and sums
-// use explicitly rounded FP64 operations (no FMA contraction), so masses and centres of mass are
-// reproducible bit for bit by any implementation that sums in the same order.
-// k_amr_reduce: one CTA walks the amr-tree from the deepest level to the root; each non-leaf
-// block sums its 8 contiguous children.
-// Both also write the FP32 records of every group of 8 siblings structure-of-arrays (x[8], y[8],
+// leaf-block node are then summed in shared memory, children in octant order, one thread per node
+// and component (mass, and mass times each coordinate).  Products and sums use explicitly rounded
+// FP64 operations (no FMA contraction), so masses and centres of mass are reproducible bit for bit by
+// any implementation that sums in the same order.
+// The amr-tree follows in the same launch: the CTA that completes the last of 8 sibling blocks (an
+// atomic count per sibling group, put back to 0 by that CTA) sums their parent from the stored records
+// and goes on to the parent's group.  No CTA waits for another, and each sum is over all 8 children in
+// octant order whoever forms it.
+// It also writes the FP32 records of every group of 8 siblings structure-of-arrays (x[8], y[8],
 // z[8], m[8]) for the paired FP32 walk: cell group g = cells 8g..8g+7, node group g = nodes
 // 1+8g..8+8g (node ids are breadth-first, so every child group starts at 1 mod 8).
 // With the FP64 records switched off (ts_tree_fp64_records) the FP64 cell records and the FP64
@@ -16,9 +19,12 @@
 // nodes are (the amr sums read them).
 //
 // Roofline: bound by GB300's FP64 rate (1/64 of FP32; HBM-bound only once that arithmetic is
-// cheap).  Per cell it reads 8 B of density and writes a 16 B FP32 record, its 16 B sibling-group
-// copy and a 32 B FP64 record (none with the FP64 records off); per leaf-block 72 + 1 internal
-// records of 16 + 16 + 32 B (16 + 16 B for the 72 with the FP64 records off).
+// cheap), and by latency on meshes of few blocks.  Per cell it reads 8 B of density and writes a 16 B
+// FP32 record, its 16 B sibling-group copy and a 32 B FP64 record (none with the FP64 records off); per
+// leaf-block 72 + 1 internal records of 16 + 16 + 32 B (16 + 16 B for the 72 with the FP64 records off).
+// 2,097,152 cells, FP64 records off: 126 us and 40 us of a second kernel for the amr-tree before, 103 us so
+// (one thread per component; the level-1 and leaf-block sums used 8 and 1 of 32 lanes); 32^3 cells: 23 us
+// and 12.5 us.
 #include <algorithm>
 
 #include "ts_internal.cuh"
@@ -31,53 +37,53 @@ __device__ __forceinline__ int morton_of(int i, int j, int k) {
     return 64 * q + 8 * o + o2;
 }
 
-struct Mom {
-    double m, sx, sy, sz;
-};
-
-__device__ __forceinline__ void mom_add(Mom& a, double m, double x, double y, double z) {
-    a.m = __dadd_rn(a.m, m);
-    a.sx = __dadd_rn(a.sx, __dmul_rn(m, x));
-    a.sy = __dadd_rn(a.sy, __dmul_rn(m, y));
-    a.sz = __dadd_rn(a.sz, __dmul_rn(m, z));
-}
-
 // node nid >= 1 is sibling (nid - 1) % 8 of node group (nid - 1) / 8; the root belongs to none
 __device__ __forceinline__ void store_soa(float* soa, int64_t g, int j, float x, float y, float z, float m) {
     float* q = soa + 32 * g + j;
     q[0] = x; q[8] = y; q[16] = z; q[24] = m;
 }
 
-__device__ __forceinline__ dbl4 store_node(float4* n32, dbl4* n64, float* soa, int nid, const Mom& a, const dbl4& cen,
-                                           bool w64 = true) {
-    double x, y, z;
-    if (a.m > 0) {
-        x = __ddiv_rn(a.sx, a.m); y = __ddiv_rn(a.sy, a.m); z = __ddiv_rn(a.sz, a.m);
-    } else {
-        x = cen.x; y = cen.y; z = cen.z;   // empty node: centre of mass := geometric centre
-    }
-    const dbl4 r{x, y, z, a.m};
-    if (w64) n64[nid] = r;
-    n32[nid] = make_float4((float)x, (float)y, (float)z, (float)a.m);
-    if (nid > 0) store_soa(soa, (nid - 1) >> 3, (nid - 1) & 7, (float)x, (float)y, (float)z, (float)a.m);
-    return r;
+// Component k (0: mass, 1..3: x, y, z) of a node's sums over its 8 children in octant order
+__device__ __forceinline__ double mom_step(double a, int k, double m, double x) {
+    return __dadd_rn(a, k ? __dmul_rn(m, x) : m);
 }
+
+// ... and of its record: the mass, or the centre of mass (of an empty node: the geometric centre)
+__device__ __forceinline__ double mom_value(double a, int k, double m, const dbl4& cen) {
+    if (k == 0) return m;
+    if (m > 0) return __ddiv_rn(a, m);
+    return k == 1 ? cen.x : k == 2 ? cen.y : cen.z;
+}
+
+// stores component k of node nid's records (mass last in each)
+__device__ __forceinline__ void store_comp(float4* n32, dbl4* n64, float* soa, int nid, int k, double v, bool w64) {
+    const int f = (k + 3) & 3;
+    if (w64) ((double*)&n64[nid])[f] = v;
+    ((float*)&n32[nid])[f] = (float)v;
+    if (nid > 0) soa[32 * (int64_t)((nid - 1) >> 3) + 8 * f + ((nid - 1) & 7)] = (float)v;
+}
+
+struct AmrDev {
+    const int* parent;   // [group] node id of the parent of sibling group g (nodes 1 + 8 g .. 8 + 8 g)
+    int* count;          // [group] blocks of the group completed in this build
+};
 
 __global__ void __launch_bounds__(512) k_blocktree(const double* __restrict__ rho, const double* __restrict__ leaf_lo,
                                                    const double* __restrict__ leaf_size, const int* __restrict__ leaf_nid,
                                                    const dbl4* __restrict__ ncen64, int nb, float4* __restrict__ cell32,
                                                    dbl4* __restrict__ cell64, float4* __restrict__ ncom32,
-                                                   dbl4* __restrict__ ncom64, float* __restrict__ cellsoa,
-                                                   float* __restrict__ ncomsoa, int full64) {
-    __shared__ double sm[512], sx[512], sy[512], sz[512];
-    __shared__ double l2m[64], l2x[64], l2y[64], l2z[64];
-    __shared__ double l1m[8], l1x[8], l1y[8], l1z[8];
+                                                   dbl4* ncom64, float* __restrict__ cellsoa,
+                                                   float* __restrict__ ncomsoa, int full64, AmrDev amr) {
+    // [component: m, x, y, z][cell or node], padded by one per 8 so that the threads that each sum 8
+    // consecutive entries hit different banks
+    __shared__ double sc[4][576], l2[4][72], l1[4][8];
     __shared__ double s_cc[3][8], s_dv;
     const int n = blockIdx.x, t = threadIdx.x;
     const int i = t & 7, j = (t >> 3) & 7, k = t >> 6;
     // The 8 cell-centre coordinates per axis and the cell volume, computed once per leaf-block (the
     // kernel is bound by GB300's FP64 rate).  x / 8 and x * 0.125 are the same exact scaling by a
     // power of two, so the results are bit-identical to lo + (i + 1/2) e / 8 and (e/8)^3.
+    const double r0 = rho[(size_t)n * TS_NCB + t];
     if (t < 24) {
         const int a = t >> 3, c = t & 7;
         s_cc[a][c] = __dadd_rn(leaf_lo[3 * n + a], __dmul_rn(__dmul_rn(c + 0.5, leaf_size[3 * n + a]), 0.125));
@@ -86,81 +92,87 @@ __global__ void __launch_bounds__(512) k_blocktree(const double* __restrict__ rh
         s_dv = __dmul_rn(__dmul_rn(__dmul_rn(ex, 0.125), __dmul_rn(ey, 0.125)), __dmul_rn(ez, 0.125));
     }
     __syncthreads();
-    const double m = __dmul_rn(rho[(size_t)n * TS_NCB + t], s_dv);
-    const double x = s_cc[0][i], y = s_cc[1][j], z = s_cc[2][k];
-    const int mt = morton_of(i, j, k);
-    sm[mt] = m; sx[mt] = x; sy[mt] = y; sz[mt] = z;
+    {
+        const int mt = morton_of(i, j, k), at = mt + (mt >> 3);
+        sc[0][at] = __dmul_rn(r0, s_dv);
+        sc[1][at] = s_cc[0][i]; sc[2][at] = s_cc[1][j]; sc[3][at] = s_cc[2][k];
+    }
     __syncthreads();
+    const int base = nb + 72 * n;
+    const int g2 = t & 63, k2 = t >> 6;   // level-2 node 8 q + o and component of this thread
+    double a2 = 0;
+    if (t < 256) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) a2 = mom_step(a2, k2, sc[0][9 * g2 + c], sc[k2][9 * g2 + c]);
+        if (k2 == 0) l2[0][g2 + (g2 >> 3)] = a2;
+    }
     // cell records in Morton order (coalesced)
     {
         const size_t id = (size_t)n * TS_NCB + t;
-        if (full64) cell64[id] = dbl4{sx[t], sy[t], sz[t], sm[t]};
-        cell32[id] = make_float4((float)sx[t], (float)sy[t], (float)sz[t], (float)sm[t]);
-        store_soa(cellsoa, (int64_t)(id >> 3), t & 7, (float)sx[t], (float)sy[t], (float)sz[t], (float)sm[t]);
-    }
-    const int base = nb + 72 * n;
-    if (t < 64) {   // level-2 node g = 8 q + o: cells 8 g .. 8 g + 7
-        Mom a{0, 0, 0, 0};
-        for (int c = 0; c < 8; ++c) mom_add(a, sm[8 * t + c], sx[8 * t + c], sy[8 * t + c], sz[8 * t + c]);
-        const int nid = base + 8 + t;
-        const dbl4 r = store_node(ncom32, ncom64, ncomsoa, nid, a, ncen64[nid], full64);
-        l2m[t] = a.m;
-        l2x[t] = r.x; l2y[t] = r.y; l2z[t] = r.z;
+        const int at = t + (t >> 3);
+        const double x = sc[1][at], y = sc[2][at], z = sc[3][at], m = sc[0][at];
+        if (full64) cell64[id] = dbl4{x, y, z, m};
+        cell32[id] = make_float4((float)x, (float)y, (float)z, (float)m);
+        store_soa(cellsoa, (int64_t)(id >> 3), t & 7, (float)x, (float)y, (float)z, (float)m);
     }
     __syncthreads();
-    if (t < 8) {    // level-1 node q: level-2 nodes 8 q .. 8 q + 7
-        Mom a{0, 0, 0, 0};
-        for (int c = 0; c < 8; ++c) mom_add(a, l2m[8 * t + c], l2x[8 * t + c], l2y[8 * t + c], l2z[8 * t + c]);
-        const int nid = base + t;
-        const dbl4 r = store_node(ncom32, ncom64, ncomsoa, nid, a, ncen64[nid], full64);
-        l1m[t] = a.m;
-        l1x[t] = r.x; l1y[t] = r.y; l1z[t] = r.z;
+    if (t < 256) {
+        const int nid = base + 8 + g2;
+        const double v = mom_value(a2, k2, l2[0][g2 + (g2 >> 3)], ncen64[nid]);
+        if (k2) l2[k2][g2 + (g2 >> 3)] = v;
+        store_comp(ncom32, ncom64, ncomsoa, nid, k2, v, full64);
     }
     __syncthreads();
-    if (t == 0) {   // the leaf-block node itself
-        Mom a{0, 0, 0, 0};
-        for (int c = 0; c < 8; ++c) mom_add(a, l1m[c], l1x[c], l1y[c], l1z[c]);
-        const int nid = leaf_nid[n];
-        store_node(ncom32, ncom64, ncomsoa, nid, a, ncen64[nid]);
-    }
-}
-
-__global__ void __launch_bounds__(256) k_amr_reduce(const int* __restrict__ order, const int* __restrict__ level_off,
-                                                    int nrounds, const dbl4* __restrict__ ncen64,
-                                                    float4* __restrict__ ncom32, dbl4* __restrict__ ncom64,
-                                                    float* __restrict__ ncomsoa) {
-    for (int r = 0; r < nrounds; ++r) {
-        for (int idx = level_off[r] + threadIdx.x; idx < level_off[r + 1]; idx += blockDim.x) {
-            const int nid = order[idx];
-            const dbl4 cen = ncen64[nid];
-            uint32_t cw = (uint32_t)cen.w;
-            const int first = (int)(cw & TS_CW_INDEX_MASK);
-            Mom a{0, 0, 0, 0};
-            for (int c = 0; c < 8; ++c) {
-                const dbl4 ch = ncom64[first + c];
-                mom_add(a, ch.w, ch.x, ch.y, ch.z);
-            }
-            store_node(ncom32, ncom64, ncomsoa, nid, a, cen);
+    if (t >= 32) return;
+    // one warp from here on: lane 4 q + k takes component k of level-1 node q
+    const int kk = t & 3, q = t >> 2;
+    double a = 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) a = mom_step(a, kk, l2[0][9 * q + c], l2[kk][9 * q + c]);
+    double v = mom_value(a, kk, __shfl_sync(0xffffffffu, a, t & ~3), ncen64[base + q]);
+    l1[kk][q] = v;
+    store_comp(ncom32, ncom64, ncomsoa, base + q, kk, v, full64);
+    __syncwarp();
+    a = 0;   // the leaf-block node (every 4 lanes form it, lanes 0..3 store it)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) a = mom_step(a, kk, l1[0][c], l1[kk][c]);
+    int nid = leaf_nid[n];
+    v = mom_value(a, kk, __shfl_sync(0xffffffffu, a, t & ~3), ncen64[nid]);
+    if (t < 4) store_comp(ncom32, ncom64, ncomsoa, nid, kk, v, true);
+    // amr ancestors completed by this block
+    while (nid > 0) {
+        const int g = (nid - 1) >> 3;
+        __threadfence();
+        __syncwarp();
+        int done = 0;
+        if (t == 0) {
+            done = atomicAdd(&amr.count[g], 1);
+            if (done == 7) amr.count[g] = 0;   // (the last arrival: ready for the next build)
         }
-        __syncthreads();
-        __threadfence_block();
+        if (__shfl_sync(0xffffffffu, done, 0) != 7) return;
+        __threadfence();
+        const double* ch = (const double*)&ncom64[1 + 8 * g];   // the 8 siblings' records (x, y, z, m)
+        double m[8], x[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {   // (through L2: other CTAs wrote them)
+            m[c] = __ldcg(ch + 4 * c + 3);
+            x[c] = __ldcg(ch + 4 * c + ((kk + 3) & 3));
+        }
+        a = 0;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) a = mom_step(a, kk, m[c], x[c]);
+        nid = amr.parent[g];
+        v = mom_value(a, kk, __shfl_sync(0xffffffffu, a, t & ~3), ncen64[nid]);
+        if (t < 4) store_comp(ncom32, ncom64, ncomsoa, nid, kk, v, true);
     }
 }
 
 cudaError_t launch_tree_build(ts_ctx* c, const double* density) {
     k_blocktree<<<c->nleaf, 512, 0, c->stream>>>(density, c->d_leaf_lo, c->d_leaf_size, c->d_leaf_nid, c->d_ncen64,
                                                  c->nb, c->d_cell32, c->d_cell64, c->d_ncom32, c->d_ncom64,
-                                                 (float*)c->d_cellsoa, (float*)c->d_ncomsoa, c->rec64 ? 1 : 0);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    // the level offsets are stored after the node ids in the same device array
-    const int nrounds = (int)c->amr_level_off.size() - 1;
-    if (nrounds > 0 && !c->amr_order.empty()) {
-        k_amr_reduce<<<1, 256, 0, c->stream>>>(c->d_amr_order, c->d_amr_order + c->amr_order.size(), nrounds,
-                                               c->d_ncen64, c->d_ncom32, c->d_ncom64, (float*)c->d_ncomsoa);
-        e = cudaGetLastError();
-    }
-    return e;
+                                                 (float*)c->d_cellsoa, (float*)c->d_ncomsoa, c->rec64 ? 1 : 0,
+                                                 AmrDev{c->d_amr_parent, c->d_amr_count});
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------------------ MPE moments

@@ -99,7 +99,9 @@ struct ts_ctx {
     int* d_leaf_nid = nullptr;       // [nleaf]
     double* d_leaf_lo = nullptr;     // [nleaf*3]
     double* d_leaf_size = nullptr;   // [nleaf*3]
-    int* d_amr_order = nullptr;      // [nb - nleaf]
+    // one buffer: the non-leaf node ids [nb - nleaf] and their offsets per round, then the parent's node
+    // id and the completed blocks (0 between builds) of every sibling group of amr nodes [(nb - 1) / 8]
+    int *d_amr_order = nullptr, *d_amr_parent = nullptr, *d_amr_count = nullptr;
     float4 *d_ncom32 = nullptr, *d_ncen32 = nullptr, *d_cell32 = nullptr;
     // FP32 positions and masses of every group of 8 siblings, structure of arrays (x[8], y[8],
     // z[8], m[8]: 8 float4 per group) for the paired walk: cells 8 g .. 8 g + 7 are cell group g,
