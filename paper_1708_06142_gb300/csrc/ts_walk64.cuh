@@ -6,13 +6,15 @@
 //   - MAC and safe-box tests run in FP32 with a guard band wider than the FP32 rounding of the
 //     coordinates; only a lane inside the band decides in FP64, by the same expressions as the scalar
 //     walk, so every decision is the FP64 one;
-//   - m / |d| and m / |d|^3 are formed by 64-bit integer arithmetic on the mantissas (pair64): an
-//     interaction takes 10 FP64 instructions (separation 3, d^2 3, sums 4);
+//   - d^2, m / |d| and m / |d|^3 are formed by 64-bit integer arithmetic on the mantissas (pair64): an
+//     interaction takes 7 FP64 instructions (separation 3, sums 4);
 //   - a leaf-cell group opened by at most 16 lanes (the mean is 11) spreads each target's 8 cells over
 //     2, 4 or 8 lanes, in a summation order that does not depend on how many lanes that is, so a
 //     target's result does not depend on the other targets of its warp.
 // 806,912-cell Plummer mesh, theta = 0.5: 67.4 ms with the scalar walk, 45.9 ms with FP64 reciprocal square
-// roots (18 instructions an interaction), 27.6 ms so; FP64 pipe 89 % busy.
+// roots (18 instructions an interaction), 27.6 ms with those in integers (10), 20.9 ms with d^2 too (7); the FP64
+// pipe is 87 % busy.  The integer forms are also the more precise ones: m / |d|^3 is within 0.51 units in the
+// last place, where the FP64 instructions give up to 4.5.
 #pragma once
 #include "ts_walk_dev.cuh"
 
@@ -24,17 +26,32 @@ __device__ __forceinline__ double pack64(unsigned long long q, int E) {
     return __longlong_as_double((long long)(((q + 512ull) >> 10) + ((unsigned long long)(unsigned)(E - 1) << 52)));
 }
 
-// mi = m / sqrt(x) and g3 = m / sqrt(x)^3 to FP64 rounding, without the FP64 pipe.  x = X 2^(2k - 62), X in
-// [2^62, 2^64); an FP32 seed of 1 / sqrt(X 2^-62) is refined twice, y (1 + e / 2) with e = 1 - X y^2 from 64-bit
-// fixed-point products: 2^-22 -> 2^-43 -> 2^-60 (Newton's iteration; the products' truncation is the last
-// term).  The mantissa of m is multiplied the same way.  Arguments whose exponents leave the normal
-// range (zero, subnormal, infinite or NaN ones among them) take the FP64 instructions.
-__device__ __forceinline__ void pair64(double x, double m, double& mi, double& g3) {
-    const unsigned long long xb = (unsigned long long)__double_as_longlong(x), mb = (unsigned long long)__double_as_longlong(m);
-    const int ex = (int)(xb >> 52), em = (int)(mb >> 52) & 0x7ff;   // (a negative x has ex > 2046)
-    const int k = (ex - 1023) >> 1;
+// |v| as a 64-bit fixed-point number F 2^(E - 1085) at the common biased exponent E >= that of v (F < 2^63; bits
+// below 2^-62 of the scale are dropped; zero and subnormal v count as 0)
+__device__ __forceinline__ unsigned long long fixed64(double v, int E) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int e = (int)(b >> 52) & 0x7ff;
+    const unsigned long long M = ((b & ((1ull << 52) - 1)) | 1ull << 52) << 10;
+    return e ? M >> min(E - e, 63) : 0ull;
+}
+
+// mi = m / |d| and g3 = m / |d|^3 to FP64 rounding, without the FP64 pipe.  |d|^2 is summed in 64-bit fixed
+// point at the scale of the largest component: X 2^(2k - 62), X in [2^62, 2^64).  An FP32 seed of
+// 1 / sqrt(X 2^-62) is refined twice, y (1 + e / 2) with e = 1 - X y^2 from fixed-point products: 2^-22 -> 2^-43 ->
+// 2^-60 (Newton's iteration; the products' truncation is the last term).  The mantissa of m is multiplied
+// the same way.  Arguments whose exponents come near the ends of the FP64 range (zero, infinite or NaN ones
+// among them) take the FP64 instructions.
+__device__ __forceinline__ void pair64(double dx, double dy, double dz, double m, double& mi, double& g3) {
+    const int E = max(max((__double2hiint(dx) >> 20) & 0x7ff, (__double2hiint(dy) >> 20) & 0x7ff),
+                      (__double2hiint(dz) >> 20) & 0x7ff);
+    const unsigned long long mb = (unsigned long long)__double_as_longlong(m);
+    const int em = (int)(mb >> 52) & 0x7ff;
     const unsigned long long one = 1ull << 52;
-    const unsigned long long X = ((xb & (one - 1)) | one) << (10 + ((ex - 1023) & 1));
+    const unsigned long long fx = fixed64(dx, E), fy = fixed64(dy, E), fz = fixed64(dz, E);
+    const unsigned long long S = __umul64hi(fx, fx) + __umul64hi(fy, fy) + __umul64hi(fz, fz);   // in [2^60, 3 2^62)
+    const int sh = S >> 62 ? 0 : 2;
+    const unsigned long long X = S << sh;
+    const int k = E - 1022 - (sh >> 1);
     float f;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"((float)(unsigned)(X >> 32) * 9.31322574615478515625e-10f));   // 2^-30
     const unsigned y0 = min(__float2uint_rn(f * 2147483648.f), 0x80000000u);                                        // 2^31 y
@@ -48,12 +65,12 @@ __device__ __forceinline__ void pair64(double x, double m, double& mi, double& g
     const unsigned long long h1 = __umul64hi(M, y), h3 = __umul64hi(M, y3);
     const int s1 = __clzll((long long)h1), s3 = __clzll((long long)h3);
     const int E1 = 1 - s1 + em - k, E3 = 2 - s3 + em - 3 * k;
-    if ((unsigned)(ex - 1) < 2046u && (unsigned)(em - 1) < 2046u && (unsigned)(E1 - 2) < 2044u && (unsigned)(E3 - 2) < 2044u) {
+    if ((unsigned)(E - 64) < 1960u && (unsigned)(em - 1) < 2046u && (unsigned)(E1 - 2) < 2044u && (unsigned)(E3 - 2) < 2044u) {
         mi = pack64(h1 << (s1 - 1), E1);
         g3 = pack64(h3 << (s3 - 1), E3);
         if ((long long)mb < 0) { mi = -mi; g3 = -g3; }
     } else {
-        const double inv = rsqrt(x);
+        const double inv = rsqrt(dx * dx + dy * dy + dz * dz);
         mi = m * inv;
         g3 = mi * (inv * inv);
     }
@@ -65,7 +82,7 @@ struct Sum64 {
 
 // one child: the terms (mi, g3 d); zero where the lane does not take it
 __device__ __forceinline__ void terms64(bool take, double dx, double dy, double dz, double m, double& mi, double& g3) {
-    pair64(take ? dx * dx + dy * dy + dz * dz : 1.0, take ? m : 1.0, mi, g3);
+    pair64(take ? dx : 1.0, dy, dz, take ? m : 1.0, mi, g3);   // (1: keeps its own cell's zero off the slow branch)
     if (!take) mi = g3 = 0.0;
 }
 
