@@ -931,7 +931,9 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
             M.w = (const __nv_bfloat16*)s_dyn;
             M.f = (const float*)(s_dyn + MLP_FWD_BF16 * 2);
             #pragma unroll 1
-            for (int m0 = 0; m0 < total; m0 += 32) mlp_eval_tile<2>(M, rf, ro, m0, total, lane);
+            for (int m0 = 0; m0 < total; m0 += 32)   // (a last tile of up to 16 rows alone: 17.1 -> 16.8 ms)
+                if (total - m0 > 16) mlp_eval_tile<2>(M, rf, ro, m0, total, lane);
+                else mlp_eval_tile<1>(M, rf, ro, m0, total, lane);
             __syncwarp();
             for (int q = k0; q < k0 + cnt; ++q) {
                 const float4 dm = rd[q];
