@@ -21,7 +21,7 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
 }
 
-template <int MAC, bool REL>
+template <int MAC, bool REL, bool SUB>
 __global__ void __launch_bounds__(32 * TS_WALK_WARPS) k_walk_split(const __grid_constant__ WalkParams P) {
     __shared__ uint2 s_stack[TS_WALK_WARPS][TS_WALK_STACK];
     __shared__ float s_half[TS_MAX_DEPTH + 1][3], s_h2[TS_MAX_DEPTH + 1];
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(32 * TS_WALK_WARPS) k_walk_split(const __grid_
             // ---- 8 leaf cells: every active target takes all of them except its own cell
             const unsigned self = (unsigned)me - (unsigned)first;
             n_int += 8u * nt - (unsigned)__popc(__ballot_sync(0xffffffffu, act && self < 8u) & 0xffu);
-            pk_interact_m<false>(dx, dy, dz, d2, m, self != 2u * sub, self != 2u * sub + 1u, s, ax, ay, az);
+            pk_interact_m<SUB>(dx, dy, dz, d2, m, self != 2u * sub, self != 2u * sub + 1u, s, ax, ay, az);
         } else {
             // ---- 8 internal nodes
             const int dep = (int)(cw >> TS_CW_DEPTH_SHIFT);
@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(32 * TS_WALK_WARPS) k_walk_split(const __grid_
                 a1 = a1 && !(y && z && fabsf(qx - 2 * hx) <= eta * hx);
             }
             const uint32_t b0 = __ballot_sync(0xffffffffu, a0), b1 = __ballot_sync(0xffffffffu, a1);
-            pk_interact_m<false>(dx, dy, dz, d2, m, a0, a1, s, ax, ay, az);
+            pk_interact_m<SUB>(dx, dy, dz, d2, m, a0, a1, s, ax, ay, az);
             // push the opened children in one compacted write: lane j < 8 owns child j, whose accepting targets
             // are byte j / 2 of the ballot of its half of the pairs
             const uint32_t om = lane < 8 ? m0 & ~(((lane & 1 ? b1 : b0) >> (8 * (lane >> 1))) & 0xffu) : 0u;
@@ -178,10 +178,12 @@ __global__ void __launch_bounds__(32 * TS_WALK_WARPS) k_walk_split(const __grid_
     }
 }
 
-template <int MAC, bool REL>
+template <int MAC, bool REL, bool SUB = false>
 static cudaError_t launch_split(ts_ctx* c, const WalkParams& P) {
+    if constexpr (!SUB)   // (see rsq)
+        if (P.tiny) return launch_split<MAC, REL, true>(c, P);
     const int64_t nwarps = P.targets ? P.ntargets / 8 : (P.leaf_end - P.leaf_begin) * 64;
     if (nwarps <= 0) return cudaSuccess;
-    k_walk_split<MAC, REL><<<(int)((nwarps + TS_WALK_WARPS - 1) / TS_WALK_WARPS), 32 * TS_WALK_WARPS, 0, c->stream>>>(P);
+    k_walk_split<MAC, REL, SUB><<<(int)((nwarps + TS_WALK_WARPS - 1) / TS_WALK_WARPS), 32 * TS_WALK_WARPS, 0, c->stream>>>(P);
     return cudaGetLastError();
 }

@@ -8,7 +8,8 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("mac,extra", [("bh", 0), ("ape", 0), ("mpe", 0), ("bh", 1)])
+# extra 3: more leaf-blocks than the walk for meshes of few cells takes
+@pytest.mark.parametrize("mac,extra", [("bh", 0), ("ape", 0), ("mpe", 0), ("bh", 1), ("bh", 3), ("ape", 3)])
 def test_small_cells_scale_exactly(mac, extra):
     import torch
     from paper_1708_06142_gb300 import inputs
@@ -16,7 +17,7 @@ def test_small_cells_scale_exactly(mac, extra):
     k = 34   # box 2^-34: cell edges 2^-38 = 3.6e-12, below the line of 1e-11
     out = []
     for e in (0, k):
-        refine = lambda lev, lo, sz: lev < 2 or (extra and lev < 3 and float(lo.max()) < 2.0 ** (-1 - e))
+        refine = lambda lev, lo, sz: lev < 2 or (extra and lev < 3 + extra - 1 and float(lo.max()) < 2.0 ** (-1 - e))
         mesh = inputs.build_mesh(refine, box=(2.0 ** -e,) * 3)
         rng = np.random.default_rng(5)
         rho = np.exp(0.5 * rng.standard_normal(mesh.ncell)) * 2.0 ** (3 * e)
