@@ -294,7 +294,9 @@ cudaError_t launch_qsums(ts_ctx* c, int nq, const double* q) {
 // f(N_H2) = 0.965 / (1 + x / b5)^2 + 0.035 / sqrt(1 + x) exp(-8.5e-4 sqrt(1 + x)), x = N_H2 / 5e14
 // (Draine & Bertoldi 1996, eq. 37), and the mean over pixels of a CO shielding factor
 // interpolated bilinearly in a caller's table over (log10 N_CO, log10 N_H2), clamped at its
-// edges.  One thread per cell; HBM-bound (12 N_PIX + 12 bytes per cell).
+// edges.  HBM traffic 12 N_PIX + 12 bytes per cell; the exponentials, logarithms and divisions of each pixel
+// bound it.  64^3 cells, N_PIX = 48: 177 us with one thread per cell, 105 us so.
+#define SHIELD_LANES 16
 __device__ __forceinline__ void lse_step(float t, float& tm, float& s);   // (mean extinction, below)
 
 struct ShieldDev {
@@ -321,23 +323,46 @@ __device__ __forceinline__ float shield_co(const ShieldDev& S, float nco, float 
     return (r0[0] * (1.f - fh) + r0[1] * fh) * (1.f - fc) + (r1[0] * (1.f - fh) + r1[1] * fh) * fc;
 }
 
+// SHIELD_LANES lanes per cell, each taking every 16th pixel, so that a cell's rows are read in 64-byte runs; the
+// partial sums meet by shuffles, the log-sum-exp about the smaller of the two optical depths.
 __global__ void __launch_bounds__(256) k_shielding(int64_t n, int npix, const float* __restrict__ cols, ShieldDev S,
                                                    float* __restrict__ out) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += stride) {
+    const int sub = threadIdx.x & (SHIELD_LANES - 1);
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x / SHIELD_LANES;
+    // (whole warps stay in the loop for the shuffles; a lane beyond the last cell repeats it and stores nothing)
+    for (int64_t c0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / SHIELD_LANES;
+         c0 - (threadIdx.x & 31) / SHIELD_LANES < n; c0 += stride) {
+        const int64_t c = c0 < n ? c0 : n - 1;
         const float* tot = cols + c * 3 * npix;
         const float* h2 = tot + npix;
         const float* co = h2 + npix;
-        float tm = S.k25 * __ldg(tot), s = 1.f, fh = 0.f, fc = 0.f;
-        for (int p = 0; p < npix; ++p) {
-            if (p) lse_step(S.k25 * __ldg(tot + p), tm, s);
+        float tm = __int_as_float(0x7f800000), s = 0.f, fh = 0.f, fc = 0.f;   // (no pixel yet: exp(-inf) adds 0)
+        for (int p = sub; p < npix; p += SHIELD_LANES) {
+            const float t = S.k25 * __ldg(tot + p);
+            if (s == 0.f) {   // the lane's first pixel (or only infinite depths so far, which add nothing)
+                tm = t;
+                s = t == __int_as_float(0x7f800000) ? 0.f : 1.f;
+            } else {
+                lse_step(t, tm, s);
+            }
             const float nh = S.k_h2 * __ldg(h2 + p);
             fh += shield_h2(nh, S.inv_b5);
             fc += S.nco ? shield_co(S, S.k_co * __ldg(co + p), nh) : 1.f;
         }
-        out[3 * c] = (tm - logf(s) + S.ln_npix) / 2.5f;
-        out[3 * c + 1] = fh / (float)npix;
-        out[3 * c + 2] = fc / (float)npix;
+#pragma unroll
+        for (int off = 1; off < SHIELD_LANES; off <<= 1) {
+            const float t2 = __shfl_xor_sync(0xffffffffu, tm, off), s2 = __shfl_xor_sync(0xffffffffu, s, off);
+            fh += __shfl_xor_sync(0xffffffffu, fh, off);
+            fc += __shfl_xor_sync(0xffffffffu, fc, off);
+            const float m = fminf(tm, t2);   // (a lane without pixels has s = 0 at an infinite depth)
+            s = (s > 0.f ? s * expf(m - tm) : s) + (s2 > 0.f ? s2 * expf(m - t2) : s2);
+            tm = m;
+        }
+        if (sub == 0 && c0 < n) {
+            out[3 * c] = (tm - logf(s) + S.ln_npix) / 2.5f;
+            out[3 * c + 1] = fh / (float)npix;
+            out[3 * c + 2] = fc / (float)npix;
+        }
     }
 }
 
@@ -357,7 +382,7 @@ cudaError_t launch_shielding(ts_ctx* c, int64_t n, int npix, const float* cols, 
     S.lh0 = (float)p->co_lg_h2[0];
     S.sh2 = d_tab ? (float)((p->co_n_h2 - 1) / (p->co_lg_h2[1] - p->co_lg_h2[0])) : 0.f;
     S.tab = d_tab;
-    const int64_t blocks = std::min<int64_t>((n + 255) / 256, 152 * 8);
+    const int64_t blocks = std::min<int64_t>((n + 256 / SHIELD_LANES - 1) / (256 / SHIELD_LANES), 152 * 8);
     k_shielding<<<(int)blocks, 256, 0, c->stream>>>(n, npix, cols, S, out);
     return cudaGetLastError();
 }
