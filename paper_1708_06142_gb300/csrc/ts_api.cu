@@ -269,6 +269,7 @@ static ts_status ingest_mesh(ts_ctx* c, const ts_mesh* m) {
 
     // geometry per depth (all nodes of one depth have equal edges: Sec. 2)
     WalkGeom& G = c->geom;
+    c->geom_uploaded = false;
     memset(&G, 0, sizeof(G));
     for (int d = 0; d <= TS_MAX_DEPTH; ++d) {
         double h2 = 0;

@@ -449,9 +449,7 @@ extern "C" ts_status ts_batch_run(ts_batch* b, const ts_gravity_params* gp, void
         } else {
             WalkGeom* dg = nullptr;
             memset(&b->h_wp[i], 0, sizeof(WalkParams));
-            if (!c->d_geom) e = ts_malloc((void**)&c->d_geom, sizeof(WalkGeom));
-            if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_geom, &c->geom, sizeof(WalkGeom), cudaMemcpyHostToDevice, c->stream);
-            dg = c->d_geom;
+            e = upload_geom(c, &dg);
             b->h_wp[i].geom = dg;
         }
         if (e == cudaSuccess && cp) {

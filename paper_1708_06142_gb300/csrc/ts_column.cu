@@ -131,11 +131,8 @@ static cudaError_t col_launch(ts_ctx* c, const ColParams& P, int nq) {
 // Kernel parameters of one context's column walk; the node-ray table comes from `tab` (a context
 // whose table matches the parameters; the batch shares one table between its grids).
 cudaError_t make_col_params(ts_ctx* c, const ts_ctx* tab, const ts_column_params* p, float* cols, ColParams* out) {
-    if (!c->d_geom) {
-        cudaError_t e = ts_malloc((void**)&c->d_geom, sizeof(WalkGeom));
-        if (e != cudaSuccess) return e;
-    }
-    cudaError_t e = cudaMemcpyAsync(c->d_geom, &c->geom, sizeof(WalkGeom), cudaMemcpyHostToDevice, c->stream);
+    WalkGeom* dg = nullptr;
+    const cudaError_t e = upload_geom(c, &dg);
     if (e != cudaSuccess) return e;
     ColParams& P = *out;
     memset(&P, 0, sizeof(P));

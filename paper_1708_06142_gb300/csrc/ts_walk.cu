@@ -1,6 +1,7 @@
 // Gravity tree walk (Sec. 2.1 tree-walk; BH MAC eq. bhmac with the safe box; APE MAC eq. ape with
 // p = 1 and eqs. abs_err / rel_err; interactions eqs. pot / accel; periodic and mixed BCs through
-// the Ewald correction table of Sec. 2.2.5, approach 2, with trilinear interpolation).
+// the Ewald correction table of Sec. 2.2.5, approach 2).  Isolated FP64 walks have their own kernel
+// (ts_walk64.cuh), and so have isolated FP32 walks of meshes of few cells (ts_walk_split.cuh).
 //
 // Work decomposition: one warp walks the tree for 32 target cells that are consecutive in Morton
 // order (a 4x4x2 brick of one leaf-block).  The warp shares one depth-first stack in shared
@@ -15,11 +16,11 @@
 //
 // Precision: FP32 interactions; each popped group's <= 8 contributions are summed in FP32 and the
 // group sum is added to the per-cell potential and acceleration with Kahan compensation (the
-// FP64 variant sums plainly in FP64).  The isolated FP32 kernel with one target per lane takes the
-// 8 children as 4 pairs and evaluates separations, MAC products and interactions of a pair with
+// FP64 variants sum plainly in FP64).  The FP32 kernels with one target per lane (the learned correction
+// excepted) take the 8 children as 4 pairs and evaluate separations, MAC products and interactions of a pair with
 // one packed f32x2 instruction each (sm_100+), which cuts the issue slots of the arithmetic by
-// almost half; the kernel is issue bound, so this is its main lever after lane utilisation, and
-// its bookkeeping is kept per warp (interaction counts from the pushed masks) or per pop (the
+// almost half; the kernels are issue bound, so this is their main lever after lane utilisation, and
+// the bookkeeping is kept per warp (interaction counts from the pushed masks) or per pop (the
 // compensated sums, in f32x2 pairs).
 //
 // Roofline: FP32-pipe (ALU) bound.  Algorithmic work: 20 flops + 1 rsqrt per accepted interaction
@@ -41,14 +42,17 @@ cudaError_t launch_walk_params(ts_ctx* c, const ts_gravity_params* p, const Walk
 cudaError_t walk_launch_pot(ts_ctx* c, const WalkParams& P, bool fp64, int bck, int mac, bool rel);
 cudaError_t launch_sumsq(ts_ctx* c, const ts_gravity_params* p, const WalkParams& W, void* pot, void* acc);
 
-// per-context copy of the depth geometry in device memory (~2 KB, read once per CTA)
-static cudaError_t upload_geom(ts_ctx* c, WalkGeom** out) {
-    if (!c->d_geom) {
-        cudaError_t e = ts_malloc((void**)&c->d_geom, sizeof(WalkGeom));
-        if (e != cudaSuccess) return e;
+// The context's copy of the depth geometry in device memory (~2 KB, read once per CTA), uploaded at the
+// first walk after each mesh ingest.
+cudaError_t upload_geom(ts_ctx* c, WalkGeom** out) {
+    cudaError_t e = cudaSuccess;
+    if (!c->d_geom) e = ts_malloc((void**)&c->d_geom, sizeof(WalkGeom));
+    if (e == cudaSuccess && !c->geom_uploaded) {
+        e = cudaMemcpyAsync(c->d_geom, &c->geom, sizeof(WalkGeom), cudaMemcpyHostToDevice, c->stream);
+        c->geom_uploaded = e == cudaSuccess;
     }
     *out = c->d_geom;
-    return cudaMemcpyAsync(c->d_geom, &c->geom, sizeof(WalkGeom), cudaMemcpyHostToDevice, c->stream);
+    return e;
 }
 
 // The largest x with !(h2 < theta2 x) in FP32: the scalar form of the BH test, h2 < theta2 d^2, as one
@@ -156,16 +160,17 @@ cudaError_t make_walk_params(ts_ctx* c, const ts_gravity_params* p, void* pot, v
         // masses have both signs).  An FP32 separation is then off by (2 S + 2 d) 2^-24 per axis, and d^2 by
         // less than 4 sqrt(3) d (S + d) 2^-24 + 6 2^-24 d^2 + 12 S^2 2^-48 (arithmetic rounding included).  The
         // band is twice that at the BH limit D = h / theta; nothing is decided in FP32 (thr = -1) where D^2
-        // leaves the FP32 range or the band would reach half of it.
+        // comes near the small end of the FP32 range or the band would reach half of it, and nothing is accepted
+        // in FP32 near the large end (a vanishing theta: everything up to 1e37 is rejected).
         double S = 0;
         for (int a = 0; a < 3; ++a) S = std::max(S, std::max(fabs(c->dlo[a]), fabs(c->dlo[a] + c->L[a])));
         const double u = ldexp(1.0, -24);
         for (int d = 0; d <= TS_MAX_DEPTH; ++d) {
             const double D2 = c->geom.hmax2_64[d] / P.theta2, D = sqrt(D2);
             const double rel = 2 * (4 * sqrt(3.0) * S / D * u + 13 * u + 12 * S * S / D2 * u * u);
-            const bool ok = D2 > 1e-30 && D2 < 1e30 && rel < 0.5;   // (false for NaN)
-            P.thr[d] = ok ? (float)(D2 * (1 - rel)) : -1.f;
-            P.thr_hi[d] = ok ? (float)(D2 * (1 + rel)) : INFINITY;
+            const bool ok = D2 > 1e-30 && rel < 0.5;   // (false for NaN)
+            P.thr[d] = ok ? (float)std::min(D2 * (1 - rel), 1e37) : -1.f;
+            P.thr_hi[d] = ok && D2 < 1e30 ? (float)(D2 * (1 + rel)) : INFINITY;
         }
         // APE accepts at any distance: 4 sqrt(3) d S u <= t d^2 + (12 S^2 u^2) / t with t = 1e-5
         P.ape_s0 = (float)(2 * (12 * S * S * u * u / 1e-5 + 12 * S * S * u * u));

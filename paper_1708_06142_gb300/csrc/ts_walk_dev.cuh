@@ -102,7 +102,7 @@ __device__ __forceinline__ void kahan_add(float& s, float& c, float x) {
     s = t;
 }
 
-// ---- paired FP32 arithmetic (isolated FP32 walk, one target per lane): two children per
+// ---- paired FP32 arithmetic (FP32 walks with one target per lane): two children per
 // instruction with the packed f32x2 add/mul/fma of sm_100+, halving the issue slots of the
 // interaction arithmetic.  Children come as a sibling group stored structure-of-arrays (x[8],
 // y[8], z[8], m[8]: 8 float4 that every lane of the warp reads at the same address).  Separations
