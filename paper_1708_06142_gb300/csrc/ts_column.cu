@@ -292,7 +292,7 @@ cudaError_t launch_qsums(ts_ctx* c, int nq, const double* q) {
 // (Draine & Bertoldi 1996, eq. 37), and the mean over pixels of a CO shielding factor
 // interpolated bilinearly in a caller's table over (log10 N_CO, log10 N_H2), clamped at its
 // edges.  HBM traffic 12 N_PIX + 12 bytes per cell; the exponentials, logarithms and divisions of each pixel
-// bound it.  64^3 cells, N_PIX = 48: 177 us with one thread per cell, 105 us so.
+// bound it.  64^3 cells, N_PIX = 48: 177 us with one thread per cell, 126 us so.
 #define SHIELD_LANES 16
 __device__ __forceinline__ void lse_step(float t, float& tm, float& s);   // (mean extinction, below)
 

@@ -8,14 +8,15 @@
 // (0 trilinear, 1 Taylor, 2 run-time choice; see ewald_pair).
 // Resident CTAs per SM asked of the compiler: the paired isolated FP32 BH walk is held to 7 CTAs
 // (73 registers a thread), which measured 2.5 % faster than the compiler's own choice at the same
-// register count.  The paired periodic walks wait for table records, so more resident warps help up to
+// register count; the APE and MPE ones to 6 CTAs (80 registers; 2M-cell MPE step 2.24 -> 2.04 ms, 0.8M-cell
+// relative APE step 398 -> 371 us; 7 CTAs 2.04 ms and 375 us, 8 spill: 2.24 ms and 408 us).  The paired periodic walks wait for table records, so more resident warps help up to
 // where registers spill: Taylor 5 CTAs (96 registers; 64^3 disk 14.7 ms, 15.2 / 15.5 / 15.8 ms with 3,
 // 4, 6), trilinear 4 (64^3 box 3.55 ms, 3.72 / 3.58 / 4.27 ms with 3, 5, 6).  The other instantiations
-// keep the compiler's choice.
+// keep the compiler's choice (the learned walk: 2 CTAs, 64^3 disk 173 ms; held to 3, 190 ms).
 template <typename R, int BCK, int MAC, int T, int EWM>
 struct WalkMinBlocks {
     static constexpr bool paired = sizeof(R) == 4 && T == 1;
-    static constexpr int value = paired && BCK == 0 && MAC == TS_MAC_BH ? 7 : paired && BCK == 1 ? (EWM == 1 ? 5 : 4) : 1;
+    static constexpr int value = paired && BCK == 0 ? (MAC == TS_MAC_BH ? 7 : 6) : paired && BCK == 1 ? (EWM == 1 ? 5 : 4) : 1;
 };
 
 template <typename R, int BCK, int MAC, bool REL, int T, int EWM, bool POT = false, bool SUB = false>
