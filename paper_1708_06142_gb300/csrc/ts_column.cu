@@ -88,12 +88,13 @@ cudaError_t launch_noderay_dense(ts_ctx* c, int nside, const int dims[3], double
 #include "ts_column_dev.cuh"
 
 template <int NQ, bool SUB>
-__global__ void __launch_bounds__(32 * TS_WALK_WARPS, ColTune<NQ>::min_ctas) k_column_walk(const __grid_constant__ ColParams P) {
-    extern __shared__ float s_map[];   // [TS_WALK_WARPS][1 + NQ][npix][32]
-    __shared__ __align__(16) float4 s_com[TS_WALK_WARPS][8];
-    __shared__ __align__(16) float4 s_cen[TS_WALK_WARPS][8];
-    __shared__ __align__(8) float2 s_q[TS_WALK_WARPS][8];
-    __shared__ uint2 s_stack[TS_WALK_WARPS][TS_WALK_STACK];
+__global__ void __launch_bounds__(32 * ColTune<NQ>::warps, ColTune<NQ>::min_ctas) k_column_walk(const __grid_constant__ ColParams P) {
+    constexpr int W = ColTune<NQ>::warps;
+    extern __shared__ float s_map[];   // [W][1 + NQ][npix][32]
+    __shared__ __align__(16) float4 s_com[W][8];
+    __shared__ __align__(16) float4 s_cen[W][8];
+    __shared__ __align__(8) float2 s_q[W][8];
+    __shared__ uint2 s_stack[W][TS_WALK_STACK];
     __shared__ float s_half[TS_MAX_DEPTH + 1][3];
     __shared__ float s_h2[TS_MAX_DEPTH + 1];
     for (int t = threadIdx.x; t <= TS_MAX_DEPTH; t += blockDim.x) {
@@ -102,25 +103,24 @@ __global__ void __launch_bounds__(32 * TS_WALK_WARPS, ColTune<NQ>::min_ctas) k_c
     }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t gw = (int64_t)blockIdx.x * TS_WALK_WARPS + warp;
+    const int64_t gw = (int64_t)blockIdx.x * W + warp;
     if (gw * 32 >= P.ncell) return;
     col_walk_warp<NQ, SUB>(P, gw, lane, s_map + (size_t)warp * (1 + NQ) * P.npix * 32, s_com[warp], s_cen[warp],
                       s_stack[warp], s_half, s_h2, s_q[warp]);
 }
-
-static size_t col_smem(const ColParams& P, int nq) { return sizeof(float) * (size_t)(1 + nq) * P.npix * 32 * TS_WALK_WARPS; }
 
 template <int NQ, bool SUB>
 static cudaError_t col_launch_t(ts_ctx* c, const ColParams& P) {
     // meshes of extremely small cells keep the functions that take subnormal arguments (see rsq)
     if constexpr (!SUB)
         if (P.tiny) return col_launch_t<NQ, true>(c, P);
-    const size_t smem = col_smem(P, NQ);
+    constexpr int W = ColTune<NQ>::warps;
+    const size_t smem = sizeof(float) * (size_t)(1 + NQ) * P.npix * 32 * W;
     const int64_t nwarps = c->ncell / 32;
-    const int grid = (int)((nwarps + TS_WALK_WARPS - 1) / TS_WALK_WARPS);
+    const int grid = (int)((nwarps + W - 1) / W);
     cudaError_t e = cudaFuncSetAttribute(k_column_walk<NQ, SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_column_walk<NQ, SUB><<<grid, 32 * TS_WALK_WARPS, smem, c->stream>>>(P);
+    k_column_walk<NQ, SUB><<<grid, 32 * W, smem, c->stream>>>(P);
     return cudaGetLastError();
 }
 

@@ -43,12 +43,16 @@ struct ColParams {
 // 27.3 ms child by child with 16-byte records of packed integers, 21.8 ms so, 20.0 ms with phi as the
 // table's fastest index and rows continued by records instead of single pixels; the maps are the same bit
 // for bit.
-// cell_pairs: pairs of leaf cells whose record loads are in flight together.  With the total map alone one
-// pair at 6 CTAs per SM is fastest (128^3: 20.0 ms; two pairs 21.4); with extra quantities shared memory
-// holds 3 CTAs, so two pairs in flight pay (64^3, 3 maps: 4.93 ms; one pair 5.4).
+// cell_pairs, node_pairs: pairs of leaf cells and of internal children whose record loads are in flight
+// together.  With the total map alone one of each at 6 CTAs of 4 warps per SM is fastest (128^3: 20.0 ms; two
+// pairs of cells 21.4, two of children 20.8).  With extra quantities the maps in shared memory leave few warps
+// on an SM, so CTAs of 2 warps, which waste less of it (10 resident warps instead of 8 with 3 maps of 48
+// pixels), and two pairs in flight pay (64^3, 3 maps: 4.86 ms with 4 warps and one pair of children, 4.48 with
+// 2 warps, 4.33 with two pairs as well).
 template <int NQ>
 struct ColTune {
-    static constexpr int cell_pairs = NQ == 0 ? 1 : 2, min_ctas = NQ == 0 ? 6 : 1;
+    static constexpr int cell_pairs = NQ == 0 ? 1 : 2, node_pairs = NQ == 0 ? 1 : 2;
+    static constexpr int min_ctas = NQ == 0 ? 6 : 1, warps = NQ == 0 ? TS_WALK_WARPS : 2;
 };
 
 // Direction angles of the bins.  theta = acos u_z and phi = atan2(y, x) come from polynomials, not
@@ -355,25 +359,38 @@ __device__ __forceinline__ void col_walk_warp(const ColParams& P, int64_t gw, in
             }
             n_mac += 8u * (unsigned)__popc(mask);
             const float thr = active ? P.thr[dep] : __int_as_float(0x7f800000);
-            // per pair of children: MAC, bins and record loads, then the scatters
+            // per NP pairs of children: MACs, bins and record loads, then the scatters
+            constexpr int NP = ColTune<NQ>::node_pairs;
 #pragma unroll 1
-            for (int j = 0; j < 8; j += 2) {
-                const float4 a = s_com_w[j], b = s_com_w[j + 1];
-                float2 dx, dy, dz, d2;
-                sep2(a, b, dx, dy, dz, d2);
-                const bool a0 = d2.x > thr && !((inside >> j) & 1u), a1 = d2.y > thr && !((inside >> (j + 1)) & 1u);
-                const unsigned b0 = __ballot_sync(0xffffffffu, a0), b1 = __ballot_sync(0xffffffffu, a1);
-                if (lane == 0) {   // the accepting lanes, parked above the stack top
-                    s_stack_w[TS_WALK_STACK - 8 + j].y = b0;
-                    s_stack_w[TS_WALK_STACK - 7 + j].y = b1;
+            for (int j0 = 0; j0 < 8; j0 += 2 * NP) {
+                float2 dx[NP], dy[NP], dz[NP], d2[NP], m[NP];
+                bool a0[NP], a1[NP], any = false;
+#pragma unroll
+                for (int u = 0; u < NP; ++u) {
+                    const int j = j0 + 2 * u;
+                    const float4 a = s_com_w[j], b = s_com_w[j + 1];
+                    sep2(a, b, dx[u], dy[u], dz[u], d2[u]);
+                    m[u] = make_float2(a.w, b.w);
+                    a0[u] = d2[u].x > thr && !((inside >> j) & 1u);
+                    a1[u] = d2[u].y > thr && !((inside >> (j + 1)) & 1u);
+                    const unsigned b0 = __ballot_sync(0xffffffffu, a0[u]), b1 = __ballot_sync(0xffffffffu, a1[u]);
+                    if (lane == 0) {   // the accepting lanes, parked above the stack top
+                        s_stack_w[TS_WALK_STACK - 8 + j].y = b0;
+                        s_stack_w[TS_WALK_STACK - 7 + j].y = b1;
+                    }
+                    any = any || a0[u] || a1[u];
                 }
-                if (a0 || a1) {
-                    ColHit<NQ> hit[2];
-                    const float2 p0 = NQ ? s_q_w[j] : zq, p1 = NQ ? s_q_w[j + 1] : zq;
-                    col_bin2<NQ, SUB>(P, a0, a1, make_float2(a.w, b.w), make_float2(p0.x, p1.x), make_float2(p0.y, p1.y), dx, dy,
-                                      dz, d2, h, hit);
-                    col_scatter<NQ>(P, mapl, hit[0]);
-                    col_scatter<NQ>(P, mapl, hit[1]);
+                if (any) {
+                    ColHit<NQ> hit[2 * NP];
+#pragma unroll
+                    for (int u = 0; u < NP; ++u) {
+                        const int j = j0 + 2 * u;
+                        const float2 p0 = NQ ? s_q_w[j] : zq, p1 = NQ ? s_q_w[j + 1] : zq;
+                        col_bin2<NQ, SUB>(P, a0[u], a1[u], m[u], make_float2(p0.x, p1.x), make_float2(p0.y, p1.y), dx[u], dy[u],
+                                          dz[u], d2[u], h, hit + 2 * u);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 2 * NP; ++u) col_scatter<NQ>(P, mapl, hit[u]);
                 }
             }
             __syncwarp();
