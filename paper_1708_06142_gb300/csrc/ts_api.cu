@@ -123,6 +123,7 @@ extern "C" ts_status ts_create(ts_ctx** out, int device, void* stream) {
 }
 
 static void free_mesh(ts_ctx* c) {
+    ++c->build_gen;
     dfree(c->d_leaf_nid); dfree(c->d_leaf_lo); dfree(c->d_leaf_size); dfree(c->d_amr_order);
     dfree(c->d_leaf_anc); dfree(c->d_bmom64); dfree(c->d_bmom32);
     free_abu(c);
@@ -431,6 +432,7 @@ extern "C" ts_status ts_tree_build(ts_ctx* c, const ts_mesh* mesh, const double*
 
 extern "C" ts_status ts_tree_fp64_records(ts_ctx* c, int32_t enabled) {
     if (!c) return ts_fail(TS_ERR_INVALID_ARG, "ts_tree_fp64_records: ctx is NULL");
+    if (c->rec64 != (enabled != 0)) ++c->build_gen;
     c->rec64 = enabled != 0;
     return TS_OK;
 }

@@ -487,7 +487,8 @@ extern "C" ts_status ts_batch_run(ts_batch* b, const ts_gravity_params* gp, void
     const int64_t acc_items = items;
     b->nitems = items;
     b->ncells = cells;
-    // graph signature: everything baked into the captured launches
+    // graph signature: everything baked into the captured launches (the tree builds and zero-mean passes
+    // hold the contexts' mesh arrays by value: their generation)
     std::vector<uint64_t> sig = {(uint64_t)(gp != nullptr), (uint64_t)(cp != nullptr), gp ? (uint64_t)gp->mac : 0,
                                  gp ? (uint64_t)gp->ewald : 0,
                                  gp ? (uint64_t)gp->zero_mean : 0, (uint64_t)npix, (uint64_t)b->chunk,
@@ -498,6 +499,7 @@ extern "C" ts_status ts_batch_run(ts_batch* b, const ts_gravity_params* gp, void
     for (int i = 0; i < n; ++i)   // (they choose kernels)
         sig.push_back((uint64_t)((gp ? b->h_wp[i].tiny : 0) | (cp ? b->h_cp[i].tiny : 0)));
     for (int i = 0; i < n; ++i) {
+        sig.push_back(b->ctx[i]->build_gen);
         sig.push_back(density ? (uint64_t)density[i] : 0);
         sig.push_back(gp ? (uint64_t)pot[i] : 0);
         if (b->mode == 1) {   // kernel arguments captured by value: every descriptor byte matters

@@ -82,6 +82,7 @@ struct ts_ctx {
     bool have_mesh = false, have_tree = false;
     bool rec64 = true;                // tree builds write the FP64 cell and in-block node records
     bool rec64_valid = false;         // the current tree has them
+    uint64_t build_gen = 0;           // changes of what a tree build's launch holds: the mesh's arrays, rec64
     int nb = 0, nleaf = 0, nint = 0, depth_max = 0;
     int64_t ncell = 0;
     int bc[3] = {0, 0, 0};
