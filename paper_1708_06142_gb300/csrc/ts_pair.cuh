@@ -25,11 +25,17 @@ __device__ __forceinline__ void ld_rec(const float4* p, float4& a, float4& b) {
 }
 
 // Minimum image of two separations at once: d - L rint(d / L), the rounding to the nearest integer by
-// adding and subtracting 1.5 * 2^23 (exact below 2^22; two packed additions where rintf needs the
-// conversion unit for each value).  An isolated axis has 1 / L = L = 0.
+// adding and subtracting 1.5 * 2^23 (exact below 2^22; additions where rintf needs the conversion unit for
+// each value).  An isolated axis has 1 / L = L = 0.  The product is rounded by itself, as in the scalar
+// walks, so that a separation of exactly half a period keeps its sign whichever way 1 / L rounds: the first
+// addition is scalar because a packed one is fused with the packed product, and then half the boxes flip
+// such pairs (column maps off by up to 80 % in pixels facing them).  The two scalar additions cost 1.4 % of
+// the 128^3 column walk (19.97 -> 20.25 ms) and 2.1 % of the 128^3 Taylor walk (15.6 -> 15.9 ms); a product with
+// subnormals flushed, which is not fused either, 1.9 % and 1.6 %.
 __device__ __forceinline__ float2 pk_image(float2 d, float2 iL, float2 nL) {
-    const float2 M = make_float2(12582912.f, 12582912.f), N = make_float2(-12582912.f, -12582912.f);
-    return __ffma2_rn(__fadd2_rn(__fadd2_rn(__fmul2_rn(d, iL), M), N), nL, d);
+    const float2 q = __fmul2_rn(d, iL);
+    const float2 r = make_float2(__fadd_rn(q.x, 12582912.f), __fadd_rn(q.y, 12582912.f));
+    return __ffma2_rn(__fadd2_rn(r, make_float2(-12582912.f, -12582912.f)), nL, d);
 }
 
 // d^2 as the scalar kernels form it, fma(dx, dx, dy dy) + dz dz with the last product rounded by
