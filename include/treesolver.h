@@ -364,7 +364,8 @@ TS_API ts_status ts_batch_destroy(ts_batch* b);
 
 /* gp: gravity parameters for all grids (or NULL: no gravity); pot_dev[i] / acc_dev[i]: float
  * outputs of grid i.  cp: column parameters (or NULL: no columns); cols_dev[i]: float
- * [ncell_i][N_PIX].  density_dev: NULL (keep the trees) or n device pointers (FP64 densities).
+ * [ncell_i][N_PIX].  density_dev: NULL (keep the trees) or n device pointers (FP64 densities); the
+ * contexts are then left as after ts_tree_build, without extra column quantities.
  * Errors: INVALID_ARG, NOT_BUILT (a context without mesh or Ewald table), UNSUPPORTED. */
 TS_API ts_status ts_batch_run(ts_batch* b, const ts_gravity_params* gp, void* const* pot_dev, void* const* acc_dev,
                               const ts_column_params* cp, float* const* cols_dev, const double* const* density_dev,

@@ -297,7 +297,6 @@ static cudaError_t batch_issue_streams(ts_batch* b, const ts_gravity_params* gp,
         cudaStream_t keep = c->stream;
         c->stream = b->wstream[k];
         if (density) e = launch_tree_build(c, density[i]);
-        if (density && e == cudaSuccess) c->rec64_valid = c->rec64;
         if (e == cudaSuccess && gp) e = launch_walk_params(c, gp, b->h_wp[i], b->bck[i], 1);
         if (e == cudaSuccess && cp) e = launch_col_params(c, b->h_cp[i]);
         if (e == cudaSuccess && gp && gp->zero_mean) e = launch_zero_mean(c, TS_PREC_FP32_KAHAN, pot[i]);
@@ -325,7 +324,6 @@ static cudaError_t batch_issue(ts_batch* b, const ts_gravity_params* gp, void* c
             cudaStream_t keep = c->stream;
             c->stream = b->stream;
             e = launch_tree_build(c, density[i]);
-            if (e == cudaSuccess) c->rec64_valid = c->rec64;
             c->stream = keep;
         }
     }
@@ -512,6 +510,12 @@ extern "C" ts_status ts_batch_run(ts_batch* b, const ts_gravity_params* gp, void
             sig.push_back((uint64_t)b->bck[i]);
         }
     }
+    if (density)   // a run (also a replay) leaves every context as ts_tree_build does
+        for (ts_ctx* c : b->ctx) {
+            c->rec64_valid = c->rec64;
+            c->bmom_prec = 0;
+            c->q_n = 0;
+        }
     cudaError_t e = cudaEventRecord(b->e0, b->stream);
     if (use_graph) {
         if (!b->gexec || sig != b->gsig) {

@@ -541,6 +541,9 @@ class Batch:
             p_den = ptrs(densities, torch.float64, nc, "density")
         _check(_lib.ts_batch_run(self._b, C.byref(gravity) if gravity is not None else None, p_pot, p_acc,
                                  C.byref(column) if column is not None else None, p_cols, p_den, int(use_graph)))
+        if densities is not None:
+            for s in self.solvers:
+                s.lq = 1
 
     def sync(self):
         out = np.zeros(5, dtype=np.int64)

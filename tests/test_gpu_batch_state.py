@@ -92,3 +92,33 @@ def test_replay_follows_another_mesh_of_as_many_cells(mode):
         # (the FP64 mean is summed in no fixed order: one FP32 rounding of the potential before the shift)
         assert float((o[0] - w[0]).abs().max()) <= 2.0 ** -22 * float(w[0].abs().max())
         assert torch.equal(o[1], w[1])
+
+
+def test_mpe_walk_and_quantities_after_a_run_with_new_densities():
+    import torch
+    from paper_1708_06142_gb300.treesolver import Batch
+    mesh = _mesh(0)
+    rho, rho2 = _rho(mesh, 4), _rho(mesh, 5)
+    ts = _solver(mesh, rho)
+    kw = dict(mac="mpe", a_lim=0.05)
+    p, a = _out(mesh)
+    ts.gravity_walk(p, a, **kw)              # moments of the first density
+    ts.column_quantities(torch.stack([rho, rho]))
+    gp = ts.gravity_params(theta=0.5)
+    b = Batch([ts])
+    for g in (False, True, True):            # direct, captured, replayed
+        rho.copy_(_rho(mesh, 6) if g else rho2)
+        torch.cuda.synchronize()
+        b.run(gp, [p], [a], densities=[rho], use_graph=g)
+        b.sync()
+        ts.gravity_walk(p, a, **kw)
+        cols = torch.empty(mesh.ncell, 48, device="cuda")
+        ts.column_walk(cols)
+        ts.sync()
+        ref = _solver(mesh, rho)
+        q, c = _out(mesh)
+        ref.gravity_walk(q, c, **kw)
+        want = torch.empty(mesh.ncell, 48, device="cuda")
+        ref.column_walk(want)
+        ref.sync()
+        assert torch.equal(p, q) and torch.equal(a, c) and torch.equal(cols, want)
