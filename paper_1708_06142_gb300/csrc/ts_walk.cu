@@ -174,7 +174,8 @@ cudaError_t make_walk_params(ts_ctx* c, const ts_gravity_params* p, void* pot, v
         }
         // APE accepts at any distance: 4 sqrt(3) d S u <= t d^2 + (12 S^2 u^2) / t with t = 1e-5
         P.ape_s0 = (float)(2 * (12 * S * S * u * u / 1e-5 + 12 * S * S * u * u));
-        P.box_tol = S < 1e30 ? (float)(8 * S * u) : INFINITY;
+        // (a domain so small that its FP32 coordinates are subnormal decides no box test in FP32)
+        P.box_tol = S > 1e-30 && S < 1e30 ? (float)(8 * S * u) : INFINITY;
         P.ncen32 = c->d_ncen32;
     }
     P.pot = pot;

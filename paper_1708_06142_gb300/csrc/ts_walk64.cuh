@@ -16,6 +16,8 @@
 // pipe is 87 % busy.  The integer forms are also the more precise ones: m / |d|^3 is within 0.51 units in the
 // last place, where the FP64 instructions give up to 4.5.
 #pragma once
+#include <float.h>
+
 #include "ts_walk_dev.cuh"
 
 #define W64_GROUPED 16   // most active lanes of a cell group whose cells are spread over lanes
@@ -139,6 +141,9 @@ __global__ void __launch_bounds__(32 * TS_WALK_WARPS) k_walk64(const __grid_cons
     const float frx = (float)rx, fry = (float)ry, frz = (float)rz;
     const float2 nrx = make_float2(-frx, -frx), nry = make_float2(-fry, -fry), nrz = make_float2(-frz, -frz);
     const float fal = (float)alim, fG = (float)G, feta = (float)eta;
+    // APE: a side of the test keeps its relative error only if its factors, and G m, are normal numbers
+    // (a subnormal one met by a large h^2 or d^4 gives a wrong result of ordinary size)
+    const bool ape32 = fabsf(fG) >= FLT_MIN && fal >= FLT_MIN;
     s_pos[warp][0][lane] = rx; s_pos[warp][1][lane] = ry; s_pos[warp][2][lane] = rz;
     s_id[warp][lane] = (int)me;
     Sum64 S{0, 0, 0, 0};
@@ -260,6 +265,10 @@ __global__ void __launch_bounds__(32 * TS_WALK_WARPS) k_walk64(const __grid_cons
             unsigned sure = 0u, may = 0u;
             const float4* sx = P.ncom_soa + 8 * ((first - 1) >> 3);
             const float tlo = P.thr[dep], thi = P.thr_hi[dep], h2f = P.geom->hmax2_32[dep];
+            const bool dep32 = ape32 && h2f >= FLT_MIN;
+            if constexpr (MAC == TS_MAC_APE) __syncwarp();   // (s_com)
+            // exactly massless (a mass below the FP32 range is 0 there too)
+            auto massless = [&](int j) { return (unsigned long long)__double_as_longlong(s_com[warp][j].w) << 1 == 0ull; };
 #pragma unroll
             for (int qq = 0; qq < 2; ++qq) {
                 const float4 X = __ldg(sx + qq), Y = __ldg(sx + 2 + qq), Z = __ldg(sx + 4 + qq), M = __ldg(sx + 6 + qq);
@@ -279,10 +288,12 @@ __global__ void __launch_bounds__(32 * TS_WALK_WARPS) k_walk64(const __grid_cons
                         } else {
                             // |d2 - v| <= 2 t v + s0 (t = 1e-5 and the cross term of the coordinate errors)
                             const float lo = fmaxf(fmaf(v, 1.f - 2e-5f, -P.ape_s0), 0.f), hi = fmaf(v, 1.f + 2e-5f, P.ape_s0);
-                            const float lhs = fG * (u ? m.y : m.x) * h2f, rl = fal * lo * lo, rh = fal * hi * hi;
+                            const float mm = u ? m.y : m.x, gm = fG * mm;
+                            const float lhs = gm * h2f, rl = fal * lo * lo, rh = fal * hi * hi;
+                            const bool ok = dep32 && (fminf(fabsf(mm), fabsf(gm)) >= FLT_MIN || (mm == 0.f && massless(4 * qq + 2 * h + u)));
                             // (a left side below 1e-30 may have underflowed: it counts as 1e-30)
-                            s = lhs >= 0.f && rl < 1e30f && fmaxf(lhs, 1e-30f) * 1.000002f < rl;
-                            y = !(lhs > 1e-30f && lhs < 1e30f && lhs * 0.999998f >= rh);
+                            s = ok && lhs >= 0.f && rl < 1e30f && fmaxf(lhs, 1e-30f) * 1.000002f < rl;
+                            y = !(ok && lhs > 1e-30f && lhs < 1e30f && lhs * 0.999998f >= rh);
                         }
                         sure |= (s ? 1u : 0u) << j;
                         may |= (y ? 1u : 0u) << j;
