@@ -442,6 +442,7 @@ extern "C" ts_status ts_batch_run(ts_batch* b, const ts_gravity_params* gp, void
         cudaError_t e = cudaSuccess;
         if (gp) {
             e = make_walk_params(c, gp, pot[i], acc[i], &b->h_wp[i], &bck);
+            b->h_wp[i].batched = 1;
             b->h_wp[i].counters = cnt + 4;   // [0..2] queues, [4..7] gravity, [8..9] column counters
             b->bck[i] = bck;
         } else {

@@ -54,6 +54,7 @@ struct WalkParams {
     uint32_t root_cw;
     uint32_t sb_depths;   // bit d: the safe-box test can change a MAC decision for nodes at depth d
     int tiny;             // 1: a squared separation of the mesh can be subnormal in FP32 (see rsq)
+    int batched;          // 1: one grid of a batch (isolated FP32 walks keep the paired kernel)
     double theta2, eta, a_lim, G, eps_rel;
     const float* a_old;
     const WalkGeom* geom;

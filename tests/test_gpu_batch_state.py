@@ -122,3 +122,27 @@ def test_mpe_walk_and_quantities_after_a_run_with_new_densities():
         ref.column_walk(want)
         ref.sync()
         assert torch.equal(p, q) and torch.equal(a, c) and torch.equal(cols, want)
+
+
+@pytest.mark.parametrize("mac", ["bh", "ape"])
+def test_both_forms_give_the_same_bits(mac):
+    import torch
+    from paper_1708_06142_gb300 import inputs
+    from paper_1708_06142_gb300.treesolver import Batch
+    meshes = [inputs.uniform_mesh(n, bc=bc) for n, bc in ((8, (0, 0, 0)), (32, (0, 0, 0)), (16, (1, 1, 1)), (16, (0, 0, 0)))]
+    rhos = [_rho(m, k) for k, m in enumerate(meshes)]
+    solvers = [_solver(m, r) for m, r in zip(meshes, rhos)]
+    solvers[2].ewald_field(16)
+    gp = solvers[0].gravity_params(mac=mac, theta=0.5, a_lim=0.05)
+    cp = solvers[0].column_params(n_side=1)
+    out = []
+    for mode in (0, 1):
+        b = Batch(solvers)
+        b.set_mode(mode, 3)
+        pots, accs = zip(*[_out(m) for m in meshes])
+        cols = [torch.empty(m.ncell, 12, device="cuda") for m in meshes]
+        b.run(gp, pots, accs, cp, cols, densities=rhos, use_graph=False)
+        b.sync()
+        out.append((*pots, *accs, *cols))
+    for x, y in zip(*out):
+        assert torch.equal(x, y)
