@@ -292,8 +292,7 @@ cudaError_t launch_qsums(ts_ctx* c, int nq, const double* q) {
 // (Draine & Bertoldi 1996, eq. 37), and the mean over pixels of a CO shielding factor
 // interpolated bilinearly in a caller's table over (log10 N_CO, log10 N_H2), clamped at its
 // edges.  HBM traffic 12 N_PIX + 12 bytes per cell; the exponentials, logarithms and divisions of each pixel
-// bound it.  64^3 cells, N_PIX = 48: 177 us with one thread per cell, 126 us so.
-#define SHIELD_LANES 16
+// bound it.
 __device__ __forceinline__ void lse_step(float t, float& tm, float& s);   // (mean extinction, below)
 
 struct ShieldDev {
@@ -320,21 +319,22 @@ __device__ __forceinline__ float shield_co(const ShieldDev& S, float nco, float 
     return (r0[0] * (1.f - fh) + r0[1] * fh) * (1.f - fc) + (r1[0] * (1.f - fh) + r1[1] * fh) * fc;
 }
 
-// SHIELD_LANES lanes per cell, each taking every 16th pixel, so that a cell's rows are read in 64-byte runs; the
-// partial sums meet by shuffles, the log-sum-exp about the smaller of the two optical depths.
+// LANES lanes per cell, each taking every LANES-th pixel, so that neighbouring lanes read runs of a cell's rows;
+// the partial sums meet by shuffles, the log-sum-exp about the smaller of the two optical depths.
+template <int LANES>
 __global__ void __launch_bounds__(256) k_shielding(int64_t n, int npix, const float* __restrict__ cols, ShieldDev S,
                                                    float* __restrict__ out) {
-    const int sub = threadIdx.x & (SHIELD_LANES - 1);
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x / SHIELD_LANES;
+    const int sub = threadIdx.x & (LANES - 1);
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x / LANES;
     // (whole warps stay in the loop for the shuffles; a lane beyond the last cell repeats it and stores nothing)
-    for (int64_t c0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / SHIELD_LANES;
-         c0 - (threadIdx.x & 31) / SHIELD_LANES < n; c0 += stride) {
+    for (int64_t c0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
+         c0 - (threadIdx.x & 31) / LANES < n; c0 += stride) {
         const int64_t c = c0 < n ? c0 : n - 1;
         const float* tot = cols + c * 3 * npix;
         const float* h2 = tot + npix;
         const float* co = h2 + npix;
         float tm = __int_as_float(0x7f800000), s = 0.f, fh = 0.f, fc = 0.f;   // (no pixel yet: exp(-inf) adds 0)
-        for (int p = sub; p < npix; p += SHIELD_LANES) {
+        for (int p = sub; p < npix; p += LANES) {
             const float t = S.k25 * __ldg(tot + p);
             if (s == 0.f) {   // the lane's first pixel (or only infinite depths so far, which add nothing)
                 tm = t;
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(256) k_shielding(int64_t n, int npix, const fl
             fc += S.nco ? shield_co(S, S.k_co * __ldg(co + p), nh) : 1.f;
         }
 #pragma unroll
-        for (int off = 1; off < SHIELD_LANES; off <<= 1) {
+        for (int off = 1; off < LANES; off <<= 1) {
             const float t2 = __shfl_xor_sync(0xffffffffu, tm, off), s2 = __shfl_xor_sync(0xffffffffu, s, off);
             fh += __shfl_xor_sync(0xffffffffu, fh, off);
             fc += __shfl_xor_sync(0xffffffffu, fc, off);
@@ -361,6 +361,17 @@ __global__ void __launch_bounds__(256) k_shielding(int64_t n, int npix, const fl
             out[3 * c + 2] = fc / (float)npix;
         }
     }
+}
+
+// Lanes per cell.  Joining the partial sums costs as much as a few pixels per lane, so short rows take few lanes;
+// long rows of few cells take more, up to where every SM has 1,024 threads.  us without a CO table, lanes 1 / 2 /
+// 4 / 8 / 16: 10^6 cells of 4 pixels 21 / 26 / 39 / 85 / 185, of 12 54 / 52 / 67 / 115 / 196, of 27 189 / 137 /
+// 139 / 176 / 252, of 48 324 / 165 / 171 / 228 / 325; 32,768 cells of 192 68 / 39 / 28 / 27 / 28, 4,096 of 192 66 / 32 /
+// 19 / 14 / 10.
+static int shield_lanes(int64_t n, int npix) {
+    int lanes = npix <= 8 ? 1 : npix <= 24 ? 2 : 4;
+    while (lanes >= 4 && lanes < 16 && n * lanes < 152 * 1024) lanes *= 2;
+    return lanes;
 }
 
 cudaError_t launch_shielding(ts_ctx* c, int64_t n, int npix, const float* cols, const ts_shield_params* p,
@@ -379,8 +390,11 @@ cudaError_t launch_shielding(ts_ctx* c, int64_t n, int npix, const float* cols, 
     S.lh0 = (float)p->co_lg_h2[0];
     S.sh2 = d_tab ? (float)((p->co_n_h2 - 1) / (p->co_lg_h2[1] - p->co_lg_h2[0])) : 0.f;
     S.tab = d_tab;
-    const int64_t blocks = std::min<int64_t>((n + 256 / SHIELD_LANES - 1) / (256 / SHIELD_LANES), 152 * 8);
-    k_shielding<<<(int)blocks, 256, 0, c->stream>>>(n, npix, cols, S, out);
+    const int lanes = shield_lanes(n, npix);
+    const int64_t blocks = std::min<int64_t>((n + 256 / lanes - 1) / (256 / lanes), 152 * 8);
+    auto* k = lanes == 1 ? k_shielding<1> : lanes == 2 ? k_shielding<2> : lanes == 4 ? k_shielding<4>
+            : lanes == 8 ? k_shielding<8> : k_shielding<16>;
+    k<<<(int)blocks, 256, 0, c->stream>>>(n, npix, cols, S, out);
     return cudaGetLastError();
 }
 
