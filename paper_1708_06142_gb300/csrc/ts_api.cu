@@ -110,6 +110,7 @@ extern "C" ts_status ts_create(ts_ctx** out, int device, void* stream) {
     if (e == cudaSuccess) e = dalloc(c->d_status, 1);
     if (e == cudaSuccess) e = dalloc(c->d_counters, 4);
     if (e == cudaSuccess) e = dalloc(c->d_reduce, 4);
+    if (e == cudaSuccess) e = dalloc(c->d_geom, 1);
     if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->d_counters, 0, 4 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaEventCreate(&c->ev0);
@@ -270,7 +271,6 @@ static ts_status ingest_mesh(ts_ctx* c, const ts_mesh* m) {
 
     // geometry per depth (all nodes of one depth have equal edges: Sec. 2)
     WalkGeom& G = c->geom;
-    c->geom_uploaded = false;
     memset(&G, 0, sizeof(G));
     for (int d = 0; d <= TS_MAX_DEPTH; ++d) {
         double h2 = 0;
@@ -399,6 +399,7 @@ static ts_status ingest_mesh(ts_ctx* c, const ts_mesh* m) {
         chk(cudaMemcpyAsync(c->d_amr_order, ord.data(), sizeof(int) * ord.size(), cudaMemcpyHostToDevice, c->stream));
         chk(cudaStreamSynchronize(c->stream));
     }
+    chk(cudaMemcpyAsync(c->d_geom, &c->geom, sizeof(WalkGeom), cudaMemcpyHostToDevice, c->stream));
     chk(cudaMemcpyAsync(c->d_ncen32, cen32.data(), sizeof(float4) * nint, cudaMemcpyHostToDevice, c->stream));
     chk(cudaMemcpyAsync(c->d_ncen64, cen64.data(), sizeof(dbl4) * nint, cudaMemcpyHostToDevice, c->stream));
     // host vectors are freed at return: wait for the copies

@@ -446,10 +446,8 @@ extern "C" ts_status ts_batch_run(ts_batch* b, const ts_gravity_params* gp, void
             b->h_wp[i].counters = cnt + 4;   // [0..2] queues, [4..7] gravity, [8..9] column counters
             b->bck[i] = bck;
         } else {
-            WalkGeom* dg = nullptr;
             memset(&b->h_wp[i], 0, sizeof(WalkParams));
-            e = upload_geom(c, &dg);
-            b->h_wp[i].geom = dg;
+            b->h_wp[i].geom = c->d_geom;
         }
         if (e == cudaSuccess && cp) {
             e = make_col_params(c, b->ctx[0], cp, cols[i], &b->h_cp[i]);

@@ -131,9 +131,6 @@ static cudaError_t col_launch(ts_ctx* c, const ColParams& P, int nq) {
 // Kernel parameters of one context's column walk; the node-ray table comes from `tab` (a context
 // whose table matches the parameters; the batch shares one table between its grids).
 cudaError_t make_col_params(ts_ctx* c, const ts_ctx* tab, const ts_column_params* p, float* cols, ColParams* out) {
-    WalkGeom* dg = nullptr;
-    const cudaError_t e = upload_geom(c, &dg);
-    if (e != cudaSuccess) return e;
     ColParams& P = *out;
     memset(&P, 0, sizeof(P));
     P.ncom = c->d_ncom32;

@@ -178,8 +178,7 @@ struct ts_ctx {
     float mlp_norm[8] = {1, 1, 1, 1, 0, 0, 0, 0};   // output scale[4], offset[4]
 
     // scratch, status and counters
-    WalkGeom* d_geom = nullptr;                 // depth geometry read by the walk kernels
-    bool geom_uploaded = false;                 // d_geom holds the current mesh's
+    WalkGeom* d_geom = nullptr;                 // depth geometry read by the walk kernels (~2 KB, of the ingested mesh)
     int* d_status = nullptr;
     unsigned long long* d_counters = nullptr;   // [0] interactions, [1] MAC tests
     double* d_reduce = nullptr;                 // FP64 reduction scratch [4]
@@ -242,7 +241,6 @@ cudaError_t launch_gravity_walk(ts_ctx* c, const ts_gravity_params* p, void* pot
 ts_status validate_gravity(ts_ctx* c, const ts_gravity_params* p);
 int ew_kind(const int bc[3]);
 float bh_threshold(float theta2, float h2);
-cudaError_t upload_geom(ts_ctx* c, WalkGeom** out);
 cudaError_t launch_zero_mean(ts_ctx* c, int precision, void* pot);
 cudaError_t launch_num_diff(ts_ctx* c, int precision, const void* pot, void* acc);
 ts_status ensure_numdiff(ts_ctx* c);

@@ -42,19 +42,6 @@ cudaError_t launch_walk_params(ts_ctx* c, const ts_gravity_params* p, const Walk
 cudaError_t walk_launch_pot(ts_ctx* c, const WalkParams& P, bool fp64, int bck, int mac, bool rel);
 cudaError_t launch_sumsq(ts_ctx* c, const ts_gravity_params* p, const WalkParams& W, void* pot, void* acc);
 
-// The context's copy of the depth geometry in device memory (~2 KB, read once per CTA), uploaded at the
-// first walk after each mesh ingest.
-cudaError_t upload_geom(ts_ctx* c, WalkGeom** out) {
-    cudaError_t e = cudaSuccess;
-    if (!c->d_geom) e = ts_malloc((void**)&c->d_geom, sizeof(WalkGeom));
-    if (e == cudaSuccess && !c->geom_uploaded) {
-        e = cudaMemcpyAsync(c->d_geom, &c->geom, sizeof(WalkGeom), cudaMemcpyHostToDevice, c->stream);
-        c->geom_uploaded = e == cudaSuccess;
-    }
-    *out = c->d_geom;
-    return e;
-}
-
 // The largest x with !(h2 < theta2 x) in FP32: the scalar form of the BH test, h2 < theta2 d^2, as one
 // comparison d^2 > x with the same decision for every d^2 (the product is monotonic in x).
 float bh_threshold(float theta2, float h2) {
@@ -74,9 +61,6 @@ float bh_threshold(float theta2, float h2) {
 // Kernel parameters of one context's walk (also used for the batched persistent kernel).
 // bck: 0 isolated, 1 correction table, 2 learned correction.
 cudaError_t make_walk_params(ts_ctx* c, const ts_gravity_params* p, void* pot, void* acc, WalkParams* out, int* bck_out) {
-    WalkGeom* dg = nullptr;
-    cudaError_t e = upload_geom(c, &dg);
-    if (e != cudaSuccess) return e;
     WalkParams& P = *out;
     memset(&P, 0, sizeof(P));
     const bool fp64 = p->precision == TS_PREC_FP64;
@@ -98,7 +82,7 @@ cudaError_t make_walk_params(ts_ctx* c, const ts_gravity_params* p, void* pot, v
     P.G = p->G;
     P.eps_rel = p->eps_rel;
     P.a_old = p->a_old_dev;
-    P.geom = dg;
+    P.geom = c->d_geom;
     // The safe box (Sec. 2.1) only matters where a target inside it could pass the MAC.  A target
     // in the eta box of a node and the node's centre of mass are at most ext = |(eta + 1) half| apart,
     // so with BH (accept iff h^2 < theta^2 d^2) and theta^2 ext^2 < h^2 an accepted node always has
