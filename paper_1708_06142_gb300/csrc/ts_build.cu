@@ -65,7 +65,7 @@ __device__ __forceinline__ void store_comp(float4* n32, dbl4* n64, float* soa, i
 
 struct AmrDev {
     const int* parent;   // [group] node id of the parent of sibling group g (nodes 1 + 8 g .. 8 + 8 g)
-    int* count;          // [group] blocks of the group completed in this build
+    unsigned* count;     // [group] blocks of the group completed in this build
 };
 
 __global__ void __launch_bounds__(512) k_blocktree(const double* __restrict__ rho, const double* __restrict__ leaf_lo,
@@ -142,15 +142,16 @@ __global__ void __launch_bounds__(512) k_blocktree(const double* __restrict__ rh
     // amr ancestors completed by this block
     while (nid > 0) {
         const int g = (nid - 1) >> 3;
-        __threadfence();
         __syncwarp();
         int done = 0;
         if (t == 0) {
-            done = atomicAdd(&amr.count[g], 1);
-            if (done == 7) amr.count[g] = 0;   // (the last arrival: ready for the next build)
+            // the barrier orders lanes 0..3's stores before this lane's fence, and the fence before its count
+            __threadfence();
+            done = (int)atomicInc(&amr.count[g], 7u);   // (the last arrival puts it back to 0 for the next build)
+            __threadfence();   // ... and orders the other blocks' stores, seen by its count, before the warp's loads
         }
         if (__shfl_sync(0xffffffffu, done, 0) != 7) return;
-        __threadfence();
+        __syncwarp();
         const double* ch = (const double*)&ncom64[1 + 8 * g];   // the 8 siblings' records (x, y, z, m)
         double m[8], x[8];
 #pragma unroll
@@ -171,7 +172,7 @@ cudaError_t launch_tree_build(ts_ctx* c, const double* density) {
     k_blocktree<<<c->nleaf, 512, 0, c->stream>>>(density, c->d_leaf_lo, c->d_leaf_size, c->d_leaf_nid, c->d_ncen64,
                                                  c->nb, c->d_cell32, c->d_cell64, c->d_ncom32, c->d_ncom64,
                                                  (float*)c->d_cellsoa, (float*)c->d_ncomsoa, c->rec64 ? 1 : 0,
-                                                 AmrDev{c->d_amr_parent, c->d_amr_count});
+                                                 AmrDev{c->d_amr_parent, (unsigned*)c->d_amr_count});
     return cudaGetLastError();
 }
 
