@@ -48,7 +48,8 @@ struct ColParams {
 // pairs of cells 21.4, two of children 20.8).  With extra quantities the maps in shared memory leave few warps
 // on an SM, so CTAs of 2 warps, which waste less of it (10 resident warps instead of 8 with 3 maps of 48
 // pixels), and two pairs in flight pay (64^3, 3 maps: 4.86 ms with 4 warps and one pair of children, 4.48 with
-// 2 warps, 4.33 with two pairs as well).
+// 2 warps, 4.33 with two pairs as well).  One extra quantity takes the same: 64^3, 2 maps of 48 pixels 3.04 ms,
+// 3.07 with 4 warps, 3.18 with one pair of each; of 12 pixels 2.42, 2.43, 2.35.
 template <int NQ>
 struct ColTune {
     static constexpr int cell_pairs = NQ == 0 ? 1 : 2, node_pairs = NQ == 0 ? 1 : 2;

@@ -13,8 +13,12 @@
 //     target's result does not depend on the other targets of its warp.
 // 806,912-cell Plummer mesh, theta = 0.5: 67.4 ms with the scalar walk, 45.9 ms with FP64 reciprocal square
 // roots (18 instructions an interaction), 27.6 ms with those in integers (10), 20.9 ms with d^2 too (7); the FP64
-// pipe is 87 % busy.  The integer forms are also the more precise ones: m / |d|^3 is within 0.51 units in the
-// last place, where the FP64 instructions give up to 4.5.
+// pipe is 87 % busy.  The integer forms are also the more precise ones: m / |d| and m / |d|^3 are within 0.56 units
+// in the last place (1/2 for the rounding; the truncated products of d^2 and of the last Newton step add up to
+// 7.5 2^-60 relative), where the FP64 instructions give up to 4.5.
+// The gain is smaller where FP32 decides less or an argument takes the FP64 instructions (348,160-cell mesh, 9.0 ms
+// in lengths of order 1, 28.4 ms with the scalar walk): lengths of 1e18 17.9 ms (nothing is accepted in FP32 from
+// h^2 / theta^2 = 1e30 on), half of the blocks massless 14.7 ms, nine tenths 19.4 ms.
 #pragma once
 #include <float.h>
 

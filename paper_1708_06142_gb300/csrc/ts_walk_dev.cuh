@@ -443,7 +443,8 @@ __device__ __forceinline__ void walk_warp(const WalkParams& P, int64_t gw, int w
     constexpr bool PKE = PK && BCK == 1;   // with the minimum image and the correction lookup
     // unrolling of the per-child loops of the scalar path: with the correction-table lookup inlined
     // into both, a 4-way unroll keeps the kernel body small enough for the instruction cache
-    // (measured on the 3P 128^3 box: Taylor 28.6 -> 24.6 ms, trilinear 67.0 -> 58.4 ms)
+    // (measured on the 3P 128^3 box with one target per lane, which the paired path has taken over: Taylor 28.6 ->
+    // 24.6 ms, trilinear 67.0 -> 58.4 ms)
     // (the paired periodic walk: its quads of children are not unrolled at all; unrolled, 18.3 ms on the
     // 64^3 Taylor disk against 16.2 ms)
     constexpr int QUAD_UNROLL = PKE ? 1 : 2;

@@ -5,9 +5,11 @@
 // long as one warp's chain of ~320 pops, with most issue slots empty.  Here lane 8 s + t handles pair s of the
 // 8 children for target t, so there are 4 times the warps, a pop is shorter, and 8 targets open fewer groups
 // than 32.  It costs more instructions a target (the bookkeeping of a pop serves 8 targets instead of 32), so
-// it is used only while the paired walk would leave the chip idle.  Walk alone, BH theta = 0.5: 16^3 cells
-// (128 warps) 70 -> 44 us, 32^3 (1,024) 110 -> 83 us (APE 28 -> 24 us), but 61,440 cells (1,920) 159 -> 178 us and
-// 64^3 (8,192) 384 -> 608 us: the line lies between.
+// it is used only while the paired walk would leave the chip idle.  Walk alone, BH, paired -> split: 16^3 cells
+// (128 warps) theta = 0.5 70 -> 44 us; 32^3 (1,024) theta = 0.4 / 0.5 / 0.8 145 -> 116, 108 -> 79, 51 -> 38 us; 36,352
+// cells (1,136) 145 -> 131, 108 -> 88, 53 -> 43 us; 47,104 (1,472) 188 -> 176, 129 -> 116, 59 -> 55 us; but 61,440
+// (1,920) theta = 0.5 159 -> 178 us and 64^3 (8,192) 384 -> 608 us.  The line, two warps per scheduler, lies below where
+// the two meet.
 // Every MAC decision is the paired walk's.
 #pragma once
 #include "ts_walk_dev.cuh"

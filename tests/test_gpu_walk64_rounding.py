@@ -56,7 +56,7 @@ def test_one_interaction(theta, unit_mass, at, seed):
                 worst_a = max(worst_a, abs(Decimal(float(a[i, k])) / (g3 * d[k]) - 1))
             else:
                 assert a[i, k] == 0.0
-    # m / d and m / d^3 to 0.54 units in the last place (1.08 u); the acceleration is one more rounding (u)
+    # m / d and m / d^3: the rounding and 7.5 2^-60 from truncated products (1.06 u); the acceleration is one more rounding (u)
     assert worst_p <= Decimal("1.1") * u, worst_p / u
     assert worst_a <= Decimal("2.1") * u, worst_a / u
 
