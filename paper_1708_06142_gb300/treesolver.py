@@ -174,8 +174,11 @@ class TreeSolver:
         self.stream = stream
         self.ncell = 0
         self._mesh_keep = None
+        self._batches = set()   # handles of the batches of this context
 
     def close(self):
+        for h in list(getattr(self, "_batches", ())):   # a batch uses its contexts' streams: it goes first
+            h.destroy()
         if self._ctx:
             _lib.ts_destroy(self._ctx)
             self._ctx = C.c_void_p()
@@ -493,6 +496,19 @@ def autotune_walk(ts: TreeSolver, pot, acc, params: TSGravityParams):
     return best.value, ms
 
 
+class _BatchHandle:
+    """A ts_batch, destroyed by its Batch or by the first of its solvers to go (garbage collection finalises
+    them in any order).  Refers to neither."""
+
+    def __init__(self):
+        self.b = C.c_void_p()
+
+    def destroy(self):
+        if self.b:
+            _lib.ts_batch_destroy(self.b)
+            self.b = C.c_void_p()
+
+
 class Batch:
     """Many independent grids (one TreeSolver each, same device) walked by one persistent kernel."""
 
@@ -500,13 +516,19 @@ class Batch:
         load()
         self.solvers = list(solvers)
         arr = (C.c_void_p * len(self.solvers))(*[s._ctx.value for s in self.solvers])
-        self._b = C.c_void_p()
-        _check(_lib.ts_batch_create(C.byref(self._b), arr, len(self.solvers)))
+        self._h = _BatchHandle()
+        _check(_lib.ts_batch_create(C.byref(self._h.b), arr, len(self.solvers)))
+        for s in self.solvers:
+            s._batches.add(self._h)
+
+    @property
+    def _b(self):
+        return self._h.b
 
     def close(self):
-        if self._b:
-            _lib.ts_batch_destroy(self._b)
-            self._b = C.c_void_p()
+        self._h.destroy()
+        for s in self.solvers:
+            s._batches.discard(self._h)
 
     def __del__(self):
         try:
